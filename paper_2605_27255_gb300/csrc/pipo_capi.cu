@@ -183,6 +183,8 @@ struct pipo_ctx {
     int32_t* samp_step = nullptr;     // draw index of the next position
     float* samp_logits = nullptr;     // [2][max_batch][V] logits of both heads
     uint32_t* presence = nullptr;     // [max_batch][presence_w] token-history bitmap
+    unsigned long long* samp_part = nullptr;  // [max_batch][slices][kSampMaxK] best keys of the vocabulary slices
+    unsigned* samp_arrived = nullptr;         // [max_batch] slices done (zero between launches)
     int presence_w = 0;
     bool prefilled = false;
     bool regular = false;             // the prefill was regular decoding (one token per backbone pass)
@@ -1208,7 +1210,7 @@ pipo_status enqueue_sample(pipo_ctx* ctx, const float* logits, int head, unsigne
     sp.head = head;
     sp.am = am;
     void* args[] = {&sp};
-    return launch_ex(ctx, (const void*)&sample_kernel, dim3(ctx->B), dim3(kSampThreads), 0, args);
+    return launch_ex(ctx, (const void*)&sample_kernel, dim3(samp_slices(c.vocab), ctx->B), dim3(kSampThreads), 0, args);
 }
 
 // One pair position of every sequence.  DECODE: the pending pair; PREFILL_*:
@@ -1219,6 +1221,8 @@ pipo_status enqueue_position(pipo_ctx* ctx, Mode mode, int j) {
     const int H = c.hidden, B = ctx->B;
     const bool bf = c.dtype == 1;
     unsigned long long* am_b = ctx->am;
+    sp.part = ctx->samp_part;
+    sp.arrived = ctx->samp_arrived;
     unsigned long long* am_d = ctx->am + c.max_batch;
 
     // pair embed + compressor (Eq. 1)
@@ -1776,6 +1780,12 @@ pipo_status pipo_set_sampler(pipo_ctx* ctx, float temperature, int32_t top_k, fl
         TRY(dalloc(ctx, &ctx->presence, (size_t)c.max_batch * ctx->presence_w * 4));
         TRY(dalloc(ctx, &ctx->samp_step, 4));
         CK(cudaMemset(ctx->presence, 0, (size_t)c.max_batch * ctx->presence_w * 4));
+    }
+    if (!ctx->samp_part)
+        TRY(dalloc(ctx, &ctx->samp_part, (size_t)c.max_batch * samp_slices(c.vocab) * kSampMaxK * 8));
+    if (!ctx->samp_arrived) {
+        TRY(dalloc(ctx, &ctx->samp_arrived, (size_t)c.max_batch * 4));
+        CK(cudaMemset(ctx->samp_arrived, 0, (size_t)c.max_batch * 4));
     }
     if (n_u > ctx->samp_nu) {
         if (ctx->samp_u) {

@@ -166,3 +166,39 @@ def test_paper_sampler_4b():
     finally:
         gpu.close()
         del w
+
+
+@pytest.mark.parametrize("V,top_k", [(24, 32), (4096, 1), (4097, 20), (8200, 32)])
+def test_vocabulary_slices(V, top_k):
+    """Vocabularies around the sampler's slice of 4096 logits, and smaller
+    than top_k: every pick is the oracle's from the GPU's own logits and
+    history.  Margin 1e-4: the fp32 penalty and temperature move a logit of
+    size < 8 by at most 2^-20, the sums of 32 exponentials by 2^-18 of their
+    mass."""
+    s = SMALL_BF16.with_(V=V)
+    w = synth.gen_weights(s, seed=11)
+    B, steps = 3, 6
+    prompts = synth.gen_prompts(B, 6, s.V, seed=4).numpy()
+    u = np.random.default_rng(V).random((steps + 1, B, 2)).astype(np.float32)
+    hist = [list(prompts[b]) for b in range(B)]
+    cfg = dict(PAPER, top_k=top_k)
+    gpu = capi.Pipo(s, w, max_batch=B, max_ctx=12, debug=True)
+    decided = 0
+    try:
+        gpu.set_sampler(u, **cfg)
+        tok, nacc = gpu.prefill(prompts)
+        for i in range(steps + 1):
+            d = gpu.debug()
+            for b in range(B):
+                for head, (lg, got) in enumerate((("logits_b", "x_b"), ("logits_d", "x_d"))):
+                    want, margin = O.sample_ex(d[lg][b], u[i, b, head], hist[b], **cfg)
+                    if margin > 1e-4:
+                        assert d[got][b] == want, (i, b, got)
+                        decided += 1
+                    if head == 0 or nacc[b]:
+                        hist[b].append(int(d[got][b]))
+            if i < steps:
+                tok, nacc = gpu.step()
+    finally:
+        gpu.close()
+    assert decided >= 24  # most of the 42 picks
