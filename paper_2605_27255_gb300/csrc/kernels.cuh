@@ -454,6 +454,9 @@ __global__ void append_rows_kernel(const float* __restrict__ qkv, int ld_qkv, in
                                    const int32_t* __restrict__ n_pos, int nseq, const float* __restrict__ rope) {
     pdl_launch();
     pdl_wait();
+    const int b = blockIdx.x, n8 = H / 8;
+    W8<T> w;
+    if ((int)threadIdx.x < n8) w.load(static_cast<const T*>(W2) + 8 * threadIdx.x);
     const int row = blockIdx.x, g = blockIdx.y, i = threadIdx.x;
     const int b = row % nseq;
     const int pos = n_pos[b] + row / nseq;
@@ -478,6 +481,8 @@ __global__ void rope_append_kernel(const float* __restrict__ qkv, int ld_qkv, fl
     pdl_launch();
     pdl_wait();
     const int b = blockIdx.x, h = blockIdx.y, i = threadIdx.x;
+    }
+    __syncthreads();
     const int pos = n_pos[b];
     const float* src = qkv + (size_t)b * ld_qkv + (size_t)h * DH;
     const int n_kv = kv.n_kv;
@@ -636,24 +641,42 @@ struct StepState {
 };
 
 // Confidence c = sigmoid(W2 . t) with t = SiLU(W1 RMSNorm([h_b; h_d])) computed
-// by the preceding GEMV; acceptance; next pending pair; counters.  grid B.
+// by the preceding GEMV; acceptance; next pending pair; counters.  grid B,
+// kAcceptThreads threads.  Latency-bound (a few KB per sequence, the last launch
+// of every step): H is a multiple of 8, so every thread takes 8 elements at
+// a time with 16-byte loads, W2 (no dependency) before the dependency wait;
+// with scalar loads in a 256-thread loop each of the H / 256 turns was a
+// round trip of its own.  Cold, with the head
+// states kept for pipo_debug_dump: 26.5 us before, 6.6 now (9B, B = 8).
+constexpr int kAcceptThreads = 512;
 template <typename T>
-__global__ void accept_kernel(const float* __restrict__ t, const void* W2, int H, float tau, int force,
-                              StepState st, const float* hb, const float* hd) {
+__global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __restrict__ t, const void* W2, int H,
+                                                                float tau, int force, StepState st, const float* hb,
+                                                                const float* hd) {
     pdl_launch();
     pdl_wait();
-    const int b = blockIdx.x;
+    const float4* t4 = reinterpret_cast<const float4*>(t + (size_t)b * H);
     float acc = 0.f;
-    for (int k = threadIdx.x; k < H; k += blockDim.x) acc += ldw<T>(W2, k) * t[(size_t)b * H + k];
+    for (int k = threadIdx.x; k < n8; k += kAcceptThreads) {
+        if (k != (int)threadIdx.x) w.load(static_cast<const T*>(W2) + 8 * k);
+        const float4 x0 = t4[2 * k], x1 = t4[2 * k + 1];
+        float f[8];
+        w.unpack(f);
+        acc += f[0] * x0.x + f[1] * x0.y + f[2] * x0.z + f[3] * x0.w + f[4] * x1.x + f[5] * x1.y + f[6] * x1.z +
+               f[7] * x1.w;
+    }
     acc = warp_sum(acc);
-    __shared__ float red[32];
+    __shared__ float red[kAcceptThreads / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) red[warp] = acc;
-    __syncthreads();
-    if (st.dbg_hb)
-        for (int k = threadIdx.x; k < H; k += blockDim.x) {
-            st.dbg_hb[(size_t)b * H + k] = hb[(size_t)b * H + k];
-            st.dbg_hd[(size_t)b * H + k] = hd[(size_t)b * H + k];
+    if (st.dbg_hb) {
+        const float4 *sb = reinterpret_cast<const float4*>(hb + (size_t)b * H),
+                     *sd = reinterpret_cast<const float4*>(hd + (size_t)b * H);
+        float4 *db = reinterpret_cast<float4*>(st.dbg_hb + (size_t)b * H),
+               *dd = reinterpret_cast<float4*>(st.dbg_hd + (size_t)b * H);
+        for (int k = threadIdx.x; k < 2 * n8; k += kAcceptThreads) {
+            db[k] = sb[k];
+            dd[k] = sd[k];
         }
     if (threadIdx.x != 0) return;
     float s = 0.f;

@@ -1301,7 +1301,7 @@ pipo_status enqueue_position(pipo_ctx* ctx, Mode mode, int j) {
         const float* hd = ctx->x2;
         void* args[] = {(void*)&tp, (void*)&w2, &Hv, &tau, &force, &st, (void*)&hb, (void*)&hd};
         return launch_ex(ctx, bf ? (const void*)&accept_kernel<bf16> : (const void*)&accept_kernel<float>, dim3(B),
-                         dim3(256), 0, args);
+                         dim3(kAcceptThreads), 0, args);
     }
 }
 
