@@ -3,7 +3,7 @@
 
 namespace pipo {
 
-void* k_pick_gemv_bf16(int nb, bool two) { return pick_gemv_t<__nv_bfloat16>(nb, two); }
+void* k_pick_block_bf16(int ru) { return pick_block_t<__nv_bfloat16>(ru); }
 void* k_pick_stream_bf16(int nb, int ru, bool rows) { return pick_stream_t<__nv_bfloat16>(nb, ru, rows); }
 
 #ifdef PIPO_TRACE

@@ -3,7 +3,7 @@
 
 namespace pipo {
 
-void* k_pick_gemv_f32(int nb, bool two) { return pick_gemv_t<float>(nb, two); }
+void* k_pick_block_f32(int ru) { return pick_block_t<float>(ru); }
 void* k_pick_stream_f32(int nb, int ru, bool rows) { return pick_stream_t<float>(nb, ru, rows); }
 
 #ifdef PIPO_TRACE

@@ -2,6 +2,7 @@
 // by k_gemv_bf16.cu and k_gemv_f32.cu).
 #pragma once
 
+#include "gemv_block.cuh"
 #include "gemv_stream.cuh"
 #include "kernel_tables.h"
 #include "kernels.cuh"
@@ -10,17 +11,9 @@ namespace pipo {
 
 constexpr int kStreamDepth = 4;  // chunks per register batch (two batches in flight)
 
-template <typename T, int NB, bool TWO>
-void* gemv_fn() { return reinterpret_cast<void*>(&gemv_kernel<T, NB, TWO>); }
-
 template <typename T>
-void* pick_gemv_t(int nb, bool two) {
-    switch (nb) {
-        case 1: return two ? gemv_fn<T, 1, true>() : gemv_fn<T, 1, false>();
-        case 2: return two ? gemv_fn<T, 2, true>() : gemv_fn<T, 2, false>();
-        case 4: return two ? gemv_fn<T, 4, true>() : gemv_fn<T, 4, false>();
-        default: return two ? gemv_fn<T, 8, true>() : gemv_fn<T, 8, false>();
-    }
+void* pick_block_t(int ru) {
+    return ru == 2 ? reinterpret_cast<void*>(&gemv_kernel<T, 2>) : reinterpret_cast<void*>(&gemv_kernel<T, 1>);
 }
 
 template <typename T, int NB, int RU>

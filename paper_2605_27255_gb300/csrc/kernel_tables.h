@@ -11,8 +11,8 @@
 namespace pipo {
 
 // k_gemv_bf16.cu / k_gemv_f32.cu: the CUDA-core GEMVs of one weight type
-void* k_pick_gemv_bf16(int nb, bool two);           // gemv_kernel<bf16, nb, two>
-void* k_pick_gemv_f32(int nb, bool two);
+void* k_pick_block_bf16(int ru);                    // gemv_kernel<bf16, ru>
+void* k_pick_block_f32(int ru);
 void* k_pick_stream_bf16(int nb, int ru, bool rows);  // gemv_rows_kernel (rows) / gemv_stream_kernel
 void* k_pick_stream_f32(int nb, int ru, bool rows);
 

@@ -11,14 +11,11 @@
 
 namespace pipo {
 
-constexpr int kThreads = 256;  // GEMV block
-constexpr int kWarps = kThreads / 32;
-
 enum Epi : int {
     EPI_STORE = 0,   // y = W x
     EPI_BIAS = 1,    // y = W x + bias
     EPI_SILU = 2,    // y = SiLU(W x)
-    EPI_RESADD = 3,  // y += W x            (residual stream; split-K: fixed-order sum)
+    EPI_RESADD = 3,  // y += W x            (residual stream)
     EPI_SWIGLU = 4,  // y = SiLU(W_2r x) * (W_2r+1 x)   (gate and up rows interleaved)
     EPI_ARGMAX = 5,  // packed (logit, -row) max per sequence; optional logits
 };
@@ -52,12 +49,9 @@ struct GemvParams {
     float* dbg;              // EPI_ARGMAX logits [B, ld_dbg] or nullptr
     int ld_dbg;
     int B;
-    int splitk;
     float eps;
     unsigned long long* zero_ptr;  // zeroed by block 0 before anything else (or nullptr)
     int zero_n;
-    float* part;         // EPI_RESADD with splitk > 1: partials [splitk][B][N]
-    unsigned* rowcnt;    // arrival counters per (batch group, row), [ceil(B/NB)][N] (zero between launches)
     // L2 warm-up of the next attention's cached pages (streaming GEMV, a
     // decode step's QKV projection; pf_k == nullptr: none).  Before its
     // dependency wait the kernel prefetches into L2 the key and value pages
@@ -238,195 +232,6 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// ---------------------------------------------------------------- GEMV
-//
-// y[b, r] = epi( sum_k W[r, k] * xin[b, k] ),  xin = staged (gathered,
-// normalised) input in shared memory, NB sequences at a time.  A warp owns one
-// (row, K-slice) task at a time and streams its weights with 128-bit
-// non-allocating loads, kU chunks in flight per lane.
-template <typename T, int NB, bool TWO>
-__global__ void __launch_bounds__(kThreads) gemv_kernel(GemvParams p) {
-    extern __shared__ float4 smem4[];
-    float* xs = reinterpret_cast<float*>(smem4);  // [NB][K]
-    __shared__ float rstd_s[NB][2];
-    constexpr int kU = 8;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int K = p.K;
-    const T* W = static_cast<const T*>(p.W);
-
-    pdl_launch();
-    pdl_wait();
-    if (p.zero_ptr && blockIdx.x == 0)
-        for (int i = threadIdx.x; i < p.zero_n; i += blockDim.x) p.zero_ptr[i] = 0ull;
-
-    const int S = p.splitk;
-    const int Ks = ((K + S * 8 - 1) / (S * 8)) * 8;
-    const int tasks = p.N * S;
-
-    for (int b0 = 0; b0 < p.B; b0 += NB) {
-        const int nb = min(NB, p.B - b0);
-        __syncthreads();
-        // ---- stage inputs
-        for (int bb = 0; bb < NB; ++bb) {
-            const int b = b0 + bb;
-            int koff = 0;
-            for (int s = 0; s < p.nseg; ++s) {
-                const Seg& sg = p.seg[s];
-                int tok = 0;
-                if (!sg.src && bb < nb) tok = sg.tok_am ? argmax_row(sg.tok_am[b]) : sg.tok[(size_t)b * sg.tok_ld];
-                for (int k = threadIdx.x; k < sg.K; k += blockDim.x) {
-                    float v = 0.f;
-                    if (bb < nb) {
-                        if (sg.src) v = sg.src[(size_t)b * sg.ld + k];
-                        else v = (tok < 0) ? ldw<T>(sg.pad, k) : ldw<T>(sg.table, (size_t)tok * sg.K + k);
-                    }
-                    xs[bb * K + koff + k] = v;
-                }
-                koff += sg.K;
-            }
-        }
-        __syncthreads();
-        // ---- RMSNorm of each segment (or of the concatenation): one warp per sum
-        const bool any_norm = p.seg[0].gamma || (p.nseg > 1 && p.seg[1].gamma);
-        if (any_norm) {
-            const int ngrp = p.joint_norm ? 1 : p.nseg;
-            for (int q = warp; q < NB * ngrp; q += kWarps) {
-                const int bb = q / ngrp, s = q % ngrp;
-                const int k0 = (s == 0) ? 0 : p.seg[0].K;
-                const int len = p.joint_norm ? K : p.seg[s].K;
-                float ss = 0.f;
-                for (int k = lane; k < len; k += 32) {
-                    float v = xs[bb * K + k0 + k];
-                    ss += v * v;
-                }
-                ss = warp_sum(ss);
-                if (lane == 0) rstd_s[bb][s] = 1.0f / sqrtf(ss / (float)len + p.eps);
-            }
-            __syncthreads();
-            for (int bb = 0; bb < NB; ++bb) {
-                for (int k = threadIdx.x; k < K; k += blockDim.x) {
-                    int s = (p.joint_norm || k < p.seg[0].K) ? 0 : 1;
-                    const Seg& sg = p.seg[s];
-                    if (!sg.gamma) continue;
-                    int kk = (p.joint_norm || s == 0) ? k : k - p.seg[0].K;
-                    xs[bb * K + k] *= rstd_s[bb][s] * ldw<T>(sg.gamma, kk);
-                }
-            }
-            __syncthreads();
-        }
-
-        // ---- rows
-        float best_v[NB];
-        int best_r[NB];
-#pragma unroll
-        for (int bb = 0; bb < NB; ++bb) { best_v[bb] = -INFINITY; best_r[bb] = 0x7fffffff; }
-
-        for (int t = blockIdx.x * kWarps + warp; t < tasks; t += gridDim.x * kWarps) {
-            const int r = t / S, s = t % S;
-            const int k0 = s * Ks, k1 = min(K, k0 + Ks);
-            float acc0[NB], acc1[NB];
-#pragma unroll
-            for (int bb = 0; bb < NB; ++bb) { acc0[bb] = 0.f; acc1[bb] = 0.f; }
-            // SwiGLU: gate row 2r and up row 2r+1 (interleaved at upload)
-            const T* w0 = W + (size_t)(TWO ? 2 * r : r) * K;
-            const T* w1 = W + (size_t)(2 * r + 1) * K;
-            for (int kb = k0 + lane * 8; kb < k1; kb += 256 * kU) {
-                W8<T> wa[kU], wb[kU];
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const int k = kb + u * 256;
-                    if (k < k1) {
-                        wa[u].load(w0 + k);
-                        if (TWO) wb[u].load(w1 + k);
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const int k = kb + u * 256;
-                    if (k < k1) {
-                        float fa[8], fb[8];
-                        wa[u].unpack(fa);
-                        if (TWO) wb[u].unpack(fb);
-#pragma unroll
-                        for (int bb = 0; bb < NB; ++bb) {
-                            const float4 x0 = *reinterpret_cast<const float4*>(xs + bb * K + k);
-                            const float4 x1 = *reinterpret_cast<const float4*>(xs + bb * K + k + 4);
-                            acc0[bb] += fa[0] * x0.x + fa[1] * x0.y + fa[2] * x0.z + fa[3] * x0.w +
-                                        fa[4] * x1.x + fa[5] * x1.y + fa[6] * x1.z + fa[7] * x1.w;
-                            if (TWO)
-                                acc1[bb] += fb[0] * x0.x + fb[1] * x0.y + fb[2] * x0.z + fb[3] * x0.w +
-                                            fb[4] * x1.x + fb[5] * x1.y + fb[6] * x1.z + fb[7] * x1.w;
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int bb = 0; bb < NB; ++bb) {
-                acc0[bb] = warp_sum(acc0[bb]);
-                if (TWO) acc1[bb] = warp_sum(acc1[bb]);
-            }
-            if (p.epi == EPI_ARGMAX) {
-#pragma unroll
-                for (int bb = 0; bb < NB; ++bb)
-                    if (acc0[bb] > best_v[bb] || (acc0[bb] == best_v[bb] && r < best_r[bb])) {
-                        best_v[bb] = acc0[bb];
-                        best_r[bb] = r;
-                    }
-                if (p.dbg && lane < nb) {
-#pragma unroll
-                    for (int bb = 0; bb < NB; ++bb)
-                        if (bb == lane) p.dbg[(size_t)(b0 + bb) * p.ld_dbg + r] = acc0[bb];
-                }
-                continue;
-            }
-            if (lane < nb) {
-#pragma unroll
-                for (int bb = 0; bb < NB; ++bb) {
-                    if (bb != lane) continue;
-                    float* yp = p.y + (size_t)(b0 + bb) * p.ldy + r;
-                    const float a = acc0[bb];
-                    switch (p.epi) {
-                        case EPI_STORE: *yp = a; break;
-                        case EPI_BIAS: *yp = a + ldw<T>(p.bias, r); break;
-                        case EPI_SILU: *yp = silu(a); break;
-                        case EPI_RESADD:
-                            if (S == 1) *yp += a;
-                            break;
-                        case EPI_SWIGLU: *yp = silu(a) * acc1[bb]; break;
-                        default: break;
-                    }
-                }
-            }
-            // split-K residual add: every slice stores its partial; the last
-            // slice of the row to arrive adds them in slice order (deterministic).
-            // CTAs reach the batch groups at different times: one counter per
-            // (group, row).
-            if (p.epi == EPI_RESADD && S > 1 && lane == 0) {
-                for (int bb = 0; bb < nb; ++bb) p.part[((size_t)s * p.B + b0 + bb) * p.N + r] = acc0[bb];
-                __threadfence();
-                unsigned* cnt = p.rowcnt + (size_t)(b0 / NB) * p.N + r;
-                const unsigned prev = atomicAdd(cnt, 1u);
-                if (prev == (unsigned)S - 1) {
-                    __threadfence();
-                    for (int bb = 0; bb < nb; ++bb) {
-                        float sum = 0.f;
-                        for (int ss = 0; ss < S; ++ss) sum += __ldcg(p.part + ((size_t)ss * p.B + b0 + bb) * p.N + r);
-                        p.y[(size_t)(b0 + bb) * p.ldy + r] += sum;
-                    }
-                    *cnt = 0u;
-                }
-            }
-        }
-        if (p.epi == EPI_ARGMAX && lane < nb) {
-#pragma unroll
-            for (int bb = 0; bb < NB; ++bb)
-                if (bb == lane && best_r[bb] != 0x7fffffff)
-                    atomicMax(p.am + b0 + bb, argmax_key(best_v[bb], best_r[bb]));
-        }
-    }
-}
-
 // ---------------------------------------------------------------- attention
 
 struct KVView {
@@ -454,9 +259,6 @@ __global__ void append_rows_kernel(const float* __restrict__ qkv, int ld_qkv, in
                                    const int32_t* __restrict__ n_pos, int nseq, const float* __restrict__ rope) {
     pdl_launch();
     pdl_wait();
-    const int b = blockIdx.x, n8 = H / 8;
-    W8<T> w;
-    if ((int)threadIdx.x < n8) w.load(static_cast<const T*>(W2) + 8 * threadIdx.x);
     const int row = blockIdx.x, g = blockIdx.y, i = threadIdx.x;
     const int b = row % nseq;
     const int pos = n_pos[b] + row / nseq;
@@ -481,8 +283,6 @@ __global__ void rope_append_kernel(const float* __restrict__ qkv, int ld_qkv, fl
     pdl_launch();
     pdl_wait();
     const int b = blockIdx.x, h = blockIdx.y, i = threadIdx.x;
-    }
-    __syncthreads();
     const int pos = n_pos[b];
     const float* src = qkv + (size_t)b * ld_qkv + (size_t)h * DH;
     const int n_kv = kv.n_kv;
@@ -654,6 +454,9 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __r
                                                                 float tau, int force, StepState st, const float* hb,
                                                                 const float* hd) {
     pdl_launch();
+    const int b = blockIdx.x, n8 = H / 8;
+    W8<T> w;
+    if ((int)threadIdx.x < n8) w.load(static_cast<const T*>(W2) + 8 * threadIdx.x);
     pdl_wait();
     const float4* t4 = reinterpret_cast<const float4*>(t + (size_t)b * H);
     float acc = 0.f;
@@ -678,6 +481,8 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __r
             db[k] = sb[k];
             dd[k] = sd[k];
         }
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
     float s = 0.f;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];

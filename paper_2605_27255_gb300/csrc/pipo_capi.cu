@@ -28,6 +28,7 @@
 #include "attn_cluster.cuh"
 #include "attn_mma.cuh"
 #include "attn_prefill.cuh"
+#include "gemv_block.cuh"
 #include "gemv_stream.cuh"
 #include "kernel_tables.h"
 #include "kernels.cuh"
@@ -115,8 +116,6 @@ struct pipo_ctx {
     float *x = nullptr, *x2 = nullptr, *qkv = nullptr, *q = nullptr, *attn = nullptr, *act = nullptr, *t = nullptr;
     float *part_o = nullptr, *part_ml = nullptr;
     unsigned* counters = nullptr;
-    float* gemv_part = nullptr;     // split-K partials of the residual-add GEMVs
-    unsigned* gemv_rowcnt = nullptr;
     unsigned long long* am = nullptr;  // [2][max_batch]
     // tensor-core projections (bf16, batch >= tc_min_b)
     bf16* tc_xb = nullptr;          // [2 * tc_bn_max][tc_kmax] bf16 activations (hi rows, lo rows)
@@ -183,9 +182,9 @@ struct pipo_ctx {
     int32_t* samp_step = nullptr;     // draw index of the next position
     float* samp_logits = nullptr;     // [2][max_batch][V] logits of both heads
     uint32_t* presence = nullptr;     // [max_batch][presence_w] token-history bitmap
+    int presence_w = 0;
     unsigned long long* samp_part = nullptr;  // [max_batch][slices][kSampMaxK] best keys of the vocabulary slices
     unsigned* samp_arrived = nullptr;         // [max_batch] slices done (zero between launches)
-    int presence_w = 0;
     bool prefilled = false;
     bool regular = false;             // the prefill was regular decoding (one token per backbone pass)
     std::vector<int32_t> h_len;
@@ -285,19 +284,17 @@ int next_pow2_le8(int b) {
 }
 
 // launch handles of the GEMV kernels of weight type T (k_gemv_*.cu)
-template <typename T>
-void* pick_gemv(int nb, bool two) {
-    return std::is_same<T, bf16>::value ? k_pick_gemv_bf16(nb, two) : k_pick_gemv_f32(nb, two);
-}
+void* pick_block(bool bf, int ru) { return bf ? k_pick_block_bf16(ru) : k_pick_block_f32(ru); }
 template <typename T>
 void* pick_stream(int nb, int ru, bool rows) {
     return std::is_same<T, bf16>::value ? k_pick_stream_bf16(nb, ru, rows) : k_pick_stream_f32(nb, ru, rows);
 }
 
-constexpr size_t kXsBudget = 100 * 1024;      // staged-input bytes per v0 GEMV block
+constexpr size_t kXsBudget = 100 * 1024;      // fp32 bytes of the longest GEMV input beyond four sequences
 // shared memory of the staged register-ring attention (the CTA's slice of
 // cached keys and values); longer slices take the register ring alone
 constexpr size_t kAttnStageMax = 160 * 1024;
+constexpr size_t kBlkSmemMax = (size_t)kBlkKMax * kBlkNB * 4 + (size_t)kBlkSeg * 32 * 4;
 constexpr size_t kStreamBudget = 200 * 1024;  // staged-input bytes per streaming GEMV block
 
 // Launch with programmatic dependent launch (decode graph) and an optional
@@ -397,13 +394,10 @@ cudaError_t set_smem_attrs(bool bf) {
                 cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamBudget);
                 if (e != cudaSuccess) return e;
             }
-    const int nbs[4] = {1, 2, 4, 8};
-    for (int i = 0; i < 4; ++i)
-        for (int two = 0; two < 2; ++two) {
-            void* f = bf ? pick_gemv<bf16>(nbs[i], two) : pick_gemv<float>(nbs[i], two);
-            cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXsBudget);
-            if (e != cudaSuccess) return e;
-        }
+    for (int ru : {1, 2}) {
+        cudaError_t e = cudaFuncSetAttribute(pick_block(bf, ru), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlkSmemMax);
+        if (e != cudaSuccess) return e;
+    }
     for (int dh : {64, 128})
         for (int g : {1, 2, 4, 8})
             for (void* f : {k_pick_attn_cluster(bf, dh, g), k_pick_attn_flat(bf, dh, g)}) {
@@ -678,6 +672,46 @@ bool tc_eligible(const pipo_ctx* ctx, const GemvParams& p) {
            p.K % kTcBK == 0 && p.K <= ctx->tc_kmax && p.K <= 4 * kPrepQ * kPrepThreads && rows >= kTcM;
 }
 
+// Clusters of KS CTAs of the row-block GEMV that can be resident at once
+// (looked up once per kernel and slice count).
+pipo_status block_clusters(pipo_ctx* ctx, const void* fn, int KS, size_t smem, int* n) {
+    const long long key = (reinterpret_cast<long long>(fn) << 4) ^ KS;
+    auto it = ctx->occ.find(key);
+    if (it != ctx->occ.end()) {
+        *n = it->second;
+        return PIPO_OK;
+    }
+    int v = ctx->sms;
+    if (KS > 1) {
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(KS);
+        lc.blockDim = dim3(kBlkThreads);
+        lc.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = KS;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        CK(cudaOccupancyMaxActiveClusters(&v, fn, &lc));
+    }
+    ctx->occ[key] = *n = std::max(1, v);
+    return PIPO_OK;
+}
+
+// Every input of the projection can be read four elements at a time: fp32
+// activations 16-byte aligned, weight-typed vectors at four elements (row
+// lengths are multiples of 8).
+bool gemv_wide_ok(const GemvParams& p) {
+    auto al = [](const void* q, size_t a) { return reinterpret_cast<uintptr_t>(q) % a == 0; };
+    for (int s = 0; s < p.nseg; ++s) {
+        const Seg& sg = p.seg[s];
+        if (!al(sg.src, 16) || sg.ld % 4 != 0 || !al(sg.table, 16) || !al(sg.pad, 16) || !al(sg.gamma, 16)) return false;
+    }
+    return true;
+}
+
 pipo_status launch_gemv(pipo_ctx* ctx, GemvParams p) {
     const bool bf = ctx->cfg.dtype == 1;
     const bool two = p.epi == EPI_SWIGLU;
@@ -698,26 +732,16 @@ pipo_status launch_gemv(pipo_ctx* ctx, GemvParams p) {
         const size_t smem = xbytes + (rows ? (size_t)p.K * ctx->esz + 16 : 0);
         return launch_ex(ctx, fn, dim3(ctx->sms * kStreamCtasPerSm), dim3(kStreamThreads), smem, args);
     }
-    int nb = next_pow2_le8(std::max(1, p.B));
-    while (nb > 1 && (size_t)nb * p.K * 4 > kXsBudget) nb >>= 1;
+    // five sequences and more: row blocks, eight sequences per weight pass
     if ((size_t)p.K * 4 > kXsBudget) return fail(ctx, PIPO_EINVAL, "GEMV input length %d too large", p.K);
-    const size_t smem = (size_t)nb * p.K * 4;
-    void* fn = bf ? pick_gemv<bf16>(nb, two) : pick_gemv<float>(nb, two);
-    const long long key = (reinterpret_cast<long long>(fn) << 1) ^ (long long)smem;
-    int per_sm;
-    auto it = ctx->occ.find(key);
-    if (it == ctx->occ.end()) {
-        CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem));
-        ctx->occ[key] = per_sm;
-    } else {
-        per_sm = it->second;
-    }
-    per_sm = std::max(1, per_sm);
-    if (p.splitk < 1) p.splitk = 1;
-    const long long tasks = (long long)p.N * p.splitk;
-    const int grid = (int)std::max(1LL, std::min<long long>((tasks + kWarps - 1) / kWarps, (long long)ctx->sms * per_sm));
-    void* args[] = {&p};
-    return launch_ex(ctx, fn, dim3(grid), dim3(kThreads), smem, args);
+    const int KS = blk_slices(p.K, (int)ctx->esz);
+    void* fn = pick_block(bf, two ? 2 : 1);
+    const size_t smem = blk_smem(p.K, (int)ctx->esz);
+    int clusters = 0;
+    TRY(block_clusters(ctx, fn, KS, smem, &clusters));
+    int wide = gemv_wide_ok(p) ? 1 : 0;
+    void* args[] = {&p, &wide};
+    return launch_ex(ctx, fn, dim3(std::min(clusters, p.N) * KS), dim3(kBlkThreads), smem, args, KS);
 }
 
 Seg act_seg(const float* src, int ld, int K, const void* gamma = nullptr) {
@@ -729,15 +753,8 @@ Seg act_seg(const float* src, int ld, int K, const void* gamma = nullptr) {
 GemvParams gemv_base(pipo_ctx* ctx, const void* W, int N, int epi, float* y, int ldy) {
     GemvParams p{};
     p.W = W; p.N = N; p.epi = epi; p.y = y; p.ldy = ldy;
-    p.B = ctx->rows > 0 ? ctx->rows : ctx->B; p.splitk = 1; p.eps = ctx->cfg.rms_eps; p.nseg = 1;
+    p.B = ctx->rows > 0 ? ctx->rows : ctx->B; p.eps = ctx->cfg.rms_eps; p.nseg = 1;
     return p;
-}
-
-int resadd_splits(pipo_ctx* ctx, int N, int K) {
-    const long long target = (long long)ctx->sms * kWarps * 2 * 4;
-    int s = (int)std::max(1LL, (target + N - 1) / N);
-    s = std::min(s, std::max(1, K / 256));
-    return s;
 }
 
 int attn_splits(const pipo_ctx* ctx, int B) {
@@ -804,8 +821,7 @@ cudaError_t set_carveouts(bool bf) {
     if (const char* ev = getenv("PIPO_CARVEOUT")) pct = atoi(ev);
     if (pct < 0) return cudaSuccess;
     std::vector<const void*> fns;
-    for (int nb : {1, 2, 4, 8})
-        for (int two = 0; two < 2; ++two) fns.push_back(bf ? pick_gemv<bf16>(nb, two) : pick_gemv<float>(nb, two));
+    for (int ru : {1, 2}) fns.push_back(pick_block(bf, ru));
     for (int nb : {1, 2, 4})
         for (int ru : {1, 2}) {
             for (bool rows : {false, true})
@@ -1147,8 +1163,6 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
     p = gemv_base(ctx, bw.Wo, H, EPI_RESADD, xr, H);
     p.seg[0] = act_seg(ctx->attn, qd, qd);
     p.K = qd;
-    p.splitk = resadd_splits(ctx, H, qd);
-    p.part = ctx->gemv_part; p.rowcnt = ctx->gemv_rowcnt;
     TRY(launch_gemv(ctx, p));
     // RMSNorm -> gate|up -> SwiGLU
     p = gemv_base(ctx, bw.Wgu, c.ffn, EPI_SWIGLU, ctx->act, c.ffn);
@@ -1159,8 +1173,6 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
     p = gemv_base(ctx, bw.Wdown, H, EPI_RESADD, xr, H);
     p.seg[0] = act_seg(ctx->act, c.ffn, c.ffn);
     p.K = c.ffn;
-    p.splitk = resadd_splits(ctx, H, c.ffn);
-    p.part = ctx->gemv_part; p.rowcnt = ctx->gemv_rowcnt;
     TRY(launch_gemv(ctx, p));
     return PIPO_OK;
 }
@@ -1209,6 +1221,8 @@ pipo_status enqueue_sample(pipo_ctx* ctx, const float* logits, int head, unsigne
     sp.u_rows = c.max_batch;
     sp.head = head;
     sp.am = am;
+    sp.part = ctx->samp_part;
+    sp.arrived = ctx->samp_arrived;
     void* args[] = {&sp};
     return launch_ex(ctx, (const void*)&sample_kernel, dim3(samp_slices(c.vocab), ctx->B), dim3(kSampThreads), 0, args);
 }
@@ -1221,8 +1235,6 @@ pipo_status enqueue_position(pipo_ctx* ctx, Mode mode, int j) {
     const int H = c.hidden, B = ctx->B;
     const bool bf = c.dtype == 1;
     unsigned long long* am_b = ctx->am;
-    sp.part = ctx->samp_part;
-    sp.arrived = ctx->samp_arrived;
     unsigned long long* am_d = ctx->am + c.max_batch;
 
     // pair embed + compressor (Eq. 1)
@@ -1691,11 +1703,6 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         TRY(dalloc(ctx, &ctx->counters, (size_t)MB * c.n_kv_heads * 4));
         CK(cudaMemset(ctx->counters, 0, (size_t)MB * c.n_kv_heads * 4));
         TRY(dalloc(ctx, &ctx->am, (size_t)2 * MB * 8));
-        const int smax = std::max(resadd_splits(ctx, H, qd), resadd_splits(ctx, H, c.ffn));
-        TRY(dalloc(ctx, &ctx->gemv_part, (size_t)smax * MR * H * 4));
-        // one counter per (batch group, row): at most MR groups
-        TRY(dalloc(ctx, &ctx->gemv_rowcnt, (size_t)MR * H * 4));
-        CK(cudaMemset(ctx->gemv_rowcnt, 0, (size_t)MR * H * 4));
         // tensor-core projections: the bf16 activation tile
         if (const char* ev = getenv("PIPO_TC_MIN_BATCH")) ctx->tc_min_b = std::max(1, atoi(ev));
         if (const char* ev = getenv("PIPO_ATTN_MMA_MIN_BATCH")) ctx->attn_mma_min_b = std::max(1, atoi(ev));
@@ -1774,18 +1781,18 @@ pipo_status pipo_set_sampler(pipo_ctx* ctx, float temperature, int32_t top_k, fl
     // off until the buffers below are in place (a failed call leaves the sampler off)
     if (ctx->samp_on) drop_graph(ctx);
     ctx->samp_on = false;
+    if (!ctx->samp_part)
+        TRY(dalloc(ctx, &ctx->samp_part, (size_t)c.max_batch * samp_slices(c.vocab) * kSampMaxK * 8));
+    if (!ctx->samp_arrived) {
+        TRY(dalloc(ctx, &ctx->samp_arrived, (size_t)c.max_batch * 4));
+        CK(cudaMemset(ctx->samp_arrived, 0, (size_t)c.max_batch * 4));
+    }
     if (!ctx->samp_logits) {
         ctx->presence_w = (c.vocab + 31) / 32;
         TRY(dalloc(ctx, &ctx->samp_logits, (size_t)2 * c.max_batch * c.vocab * 4));
         TRY(dalloc(ctx, &ctx->presence, (size_t)c.max_batch * ctx->presence_w * 4));
         TRY(dalloc(ctx, &ctx->samp_step, 4));
         CK(cudaMemset(ctx->presence, 0, (size_t)c.max_batch * ctx->presence_w * 4));
-    }
-    if (!ctx->samp_part)
-        TRY(dalloc(ctx, &ctx->samp_part, (size_t)c.max_batch * samp_slices(c.vocab) * kSampMaxK * 8));
-    if (!ctx->samp_arrived) {
-        TRY(dalloc(ctx, &ctx->samp_arrived, (size_t)c.max_batch * 4));
-        CK(cudaMemset(ctx->samp_arrived, 0, (size_t)c.max_batch * 4));
     }
     if (n_u > ctx->samp_nu) {
         if (ctx->samp_u) {
@@ -2261,7 +2268,7 @@ pipo_status op_lm_head_impl(pipo_ctx& op, int32_t dtype, const void* d_E, int32_
     p.dbg = d_logits;
     p.ld_dbg = V;
     p.B = B;
-    p.splitk = 1;
+   
     p.nseg = 1;
     p.eps = eps;
     p.seg[0] = act_seg(d_h, H, H, d_gamma);
@@ -2286,7 +2293,7 @@ pipo_status op_gemv_impl(pipo_ctx& op, int32_t dtype, int32_t mode, const void* 
     p.y = d_y;
     p.ldy = N;
     p.B = B;
-    p.splitk = 1;
+   
     p.nseg = 1;
     p.seg[0] = act_seg(d_x, K, K);
     return launch_gemv(ctx, p);
@@ -2377,7 +2384,7 @@ pipo_status pipo_op_gemv_chain(int32_t dtype, int32_t mode, const void* const* d
     pipo_status st = op_setup(op, dtype, stream);
     GemvParams p{};
     p.N = N; p.K = K; p.epi = mode == 1 ? EPI_SWIGLU : EPI_STORE; p.y = d_y; p.ldy = N; p.B = B;
-    p.splitk = 1; p.nseg = 1; p.seg[0] = act_seg(d_x, K, K);
+    p.nseg = 1; p.seg[0] = act_seg(d_x, K, K);
     for (int i = 0; st == PIPO_OK && i < count; ++i) {
         p.W = d_Ws[i];
         st = launch_gemv(ctx, p);
@@ -2423,7 +2430,7 @@ pipo_status pipo_op_gemm_tc(int32_t mode, const void* d_W, int32_t N, int32_t K,
         } else {
             GemvParams p{};
             p.W = d_W; p.N = N; p.K = K; p.epi = mode == 1 ? EPI_SWIGLU : EPI_STORE;
-            p.y = d_y; p.ldy = N; p.B = B; p.splitk = 1; p.nseg = 1;
+            p.y = d_y; p.ldy = N; p.B = B; p.nseg = 1;
             p.seg[0] = act_seg(d_x, K, K);
             st = launch_gemm_tc(ctx, p, static_cast<bf16*>(d_scratch), splits, B);
         }
@@ -2455,7 +2462,7 @@ pipo_status pipo_op_gemm_tc_norm(int32_t mode, const void* d_W, int32_t N, const
         } else {
             GemvParams p{};
             p.W = d_W; p.N = N; p.K = K; p.epi = mode == 1 ? EPI_SWIGLU : EPI_STORE;
-            p.y = d_y; p.ldy = N; p.B = B; p.splitk = 1; p.eps = eps;
+            p.y = d_y; p.ldy = N; p.B = B; p.eps = eps;
             p.nseg = two ? 2 : 1;
             p.joint_norm = joint ? 1 : 0;
             p.seg[0] = act_seg(d_x0, K0, K0, d_gamma0);
