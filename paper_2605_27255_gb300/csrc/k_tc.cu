@@ -1,6 +1,7 @@
 // tcgen05 tensor-core projection kernels (a translation unit of its own).
 #include "kernel_tables.h"
 #include "tcgen05_gemm.cuh"
+#include "tcgen05_pair.cuh"
 
 namespace pipo {
 
@@ -39,6 +40,11 @@ void* pick_tcf_v(int bh) {
 void* k_pick_tcv(int bh, bool deep, bool fused) {
     if (fused) return deep ? pick_tcf_v<true>(bh) : pick_tcf_v<false>(bh);
     return deep ? pick_tc_v<true>(bh) : pick_tc_v<false>(bh);
+}
+
+void* k_pick_pair(int nt) {
+    return nt <= 128 ? reinterpret_cast<void*>(&gemm_pair_kernel<128>)
+                     : reinterpret_cast<void*>(&gemm_pair_kernel<kPairMaxN>);
 }
 
 void* k_pick_prep_bf16() { return reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16>); }

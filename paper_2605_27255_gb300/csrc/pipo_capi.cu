@@ -35,6 +35,7 @@
 #include "pipo.h"
 #include "sampler.cuh"
 #include "tcgen05_gemm.cuh"
+#include "tcgen05_pair.cuh"
 
 using namespace pipo;
 using bf16 = __nv_bfloat16;
@@ -294,6 +295,8 @@ constexpr size_t kXsBudget = 100 * 1024;      // fp32 bytes of the longest GEMV 
 // shared memory of the staged register-ring attention (the CTA's slice of
 // cached keys and values); longer slices take the register ring alone
 constexpr size_t kAttnStageMax = 160 * 1024;
+constexpr int kMaxPrefillRows = 2048;         // rows of a prefill chunk (PIPO_PREFILL_ROWS)
+constexpr size_t kPairSmemMax = 208 * 1024;   // stages of the CTA-pair GEMM (one CTA per SM)
 constexpr size_t kBlkSmemMax = (size_t)kBlkKMax * kBlkNB * 4 + (size_t)kBlkSeg * 32 * 4;
 constexpr size_t kStreamBudget = 200 * 1024;  // staged-input bytes per streaming GEMV block
 
@@ -425,6 +428,11 @@ cudaError_t set_smem_attrs(bool bf) {
                                                                  : cudaClusterSchedulingPolicyLoadBalancing);
                     if (e != cudaSuccess) return e;
                 }
+    if (bf)
+        for (int nt : {128, kPairMaxN}) {
+            cudaError_t e = cudaFuncSetAttribute(k_pick_pair(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemMax);
+            if (e != cudaSuccess) return e;
+        }
     return cudaSuccess;
 }
 
@@ -480,7 +488,8 @@ pipo_status make_tmap_x(pipo_ctx* ctx, CUtensorMap* tm, const float* base, int K
     return PIPO_OK;
 }
 
-int tc_bn(int B) { return B <= 16 ? 16 : B <= 32 ? 32 : B <= 64 ? 64 : 128; }
+// rows of the activation buffers behind a batch of B: the box height up to 32
+int tc_bn(int B) { return B <= 16 ? 16 : B <= 32 ? 32 : B <= 64 ? 64 : B <= 128 ? 128 : B; }
 
 // resident CTAs per SM of the tensor-core GEMM at this BN (shared memory bound)
 int tc_ctas_per_sm(int bn, bool deep = false, bool fused = false) {
@@ -602,11 +611,100 @@ int tc_fused_max_bh() {
     return v;
 }
 
+// CTA pairs of the CTA-pair GEMM that can be resident at once on the current
+// device (cached).
+int pair_max_clusters(int nt, size_t smem) {
+    static std::mutex mu;
+    static std::map<long long, int> cache;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
+    const long long key = ((long long)dev << 40) | ((long long)(nt <= 128) << 32) | (long long)smem;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(2);
+    lc.blockDim = dim3(kPairThreads);
+    lc.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_pick_pair(nt), &lc) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    cache[key] = n;
+    return n;
+}
+
+// Launch plan of the CTA-pair GEMM: positions per tile, stages, pairs.  The R
+// positions are cut into equal tiles whose width makes the persistent pairs'
+// rounds shortest in total.  A 64-wide K block of a tile takes 4 NT
+// tensor-core clocks, and the 16 KB + 128 NT bytes a CTA loads for it arrive
+// at about 48 bytes per clock: 2.7 (NT + 128) clocks, the larger of the two up
+// to NT = 256.
+struct PairPlan {
+    int NT, ST, pairs;
+    size_t smem;
+};
+PairPlan pair_plan(int sms, int rows, int R) {
+    const int mt = (rows + kPairM - 1) / kPairM, pairs = std::max(1, sms / 2);
+    PairPlan pl{};
+    long long best = -1;
+    for (int nt = 32; nt <= kPairMaxN; nt += 32) {
+        const long long tiles = (long long)mt * ((R + nt - 1) / nt), cost = (tiles + pairs - 1) / pairs * (nt + 128);
+        if (best < 0 || cost <= best) { best = cost; pl.NT = nt; }
+    }
+    pl.ST = kPairMaxStages;
+    while (pl.ST > 2 && pair_smem(pl.NT, pl.ST) > kPairSmemMax) --pl.ST;
+    pl.smem = pair_smem(pl.NT, pl.ST);
+    const int tiles = mt * ((R + pl.NT - 1) / pl.NT);
+    pl.pairs = std::min(tiles, std::max(1, pair_max_clusters(pl.NT, pl.smem)));
+    return pl;
+}
+
+// Projection of a prefill chunk of more than 128 rows: bf16 hi and lo rows
+// from prep_bf16_kernel, then the CTA-pair GEMM.
+pipo_status launch_gemm_pair(pipo_ctx* ctx, const GemvParams& p, bf16* xb) {
+    if (p.epi == EPI_ARGMAX) return fail(ctx, PIPO_EINVAL, "argmax of %d rows on the CTA-pair GEMM", p.B);
+    const int ru = p.epi == EPI_SWIGLU ? 2 : 1, rows = p.N * ru;
+    const PairPlan pl = pair_plan(ctx->sms, rows, p.B);
+    PairParams q{};
+    q.t.rows = rows; q.t.K = p.K; q.t.B = p.B; q.t.ru = ru; q.t.epi = p.epi;
+    q.t.y = p.y; q.t.ldy = p.ldy; q.t.bias = p.bias;
+    q.NT = pl.NT;
+    q.ST = pl.ST;
+    q.tiles_n = (p.B + pl.NT - 1) / pl.NT;
+    q.tiles = (rows + kPairM - 1) / kPairM * q.tiles_n;
+    CUtensorMap tmW, tmX;
+    TRY(make_tmap(ctx, &tmW, p.W, p.K, rows, kTcM));
+    TRY(make_tmap(ctx, &tmX, xb, p.K, 2 * p.B, pl.NT / 2));
+    {
+        GemvParams pp = p;
+        int bh = p.B;
+        void* args[] = {&pp, &xb, &bh};
+        ctx->prof_kind = 2;
+        ctx->prof_bytes = 0.0;
+        ctx->launch_prep = true;
+        TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16()), dim3(p.B), dim3(kPrepThreads), 0, args));
+    }
+    void* args[] = {&tmW, &tmX, &q};
+    ctx->prof_kind = 0;
+    ctx->prof_bytes = (double)rows * p.K * 2;
+    return launch_ex(ctx, k_pick_pair(pl.NT), dim3(2 * pl.pairs), dim3(kPairThreads), pl.smem, args, 2);
+}
+
 // Projection on the tensor cores: the fused GEMM, or bf16 activations from
 // prep_bf16_kernel and then the tcgen05 GEMM.  Eligible: bf16 weights,
-// K % 64 == 0, rows >= 128, B <= 128.  x_rows: rows behind each activation
+// K % 64 == 0, rows >= 128.  x_rows: rows behind each activation
 // pointer (the tensor maps read no further; at least BH for box-sized maps).
 pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int splits_req, int x_rows) {
+    if (p.B > 128) return launch_gemm_pair(ctx, p, xb);
     const int ru = p.epi == EPI_SWIGLU ? 2 : 1;
     const int rows = p.N * ru, bn = tc_bn(p.B), tiles = (rows + kTcM - 1) / kTcM, nkb = p.K / kTcBK;
     const bool fused = tcf_eligible(p) && !tc_prep_forced() && x_rows >= bn && bn <= tc_fused_max_bh();
@@ -668,7 +766,10 @@ pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int spl
 
 bool tc_eligible(const pipo_ctx* ctx, const GemvParams& p) {
     const int rows = p.N * (p.epi == EPI_SWIGLU ? 2 : 1);
-    return ctx->cfg.dtype == 1 && ctx->tc_xb && p.B >= ctx->tc_min_b && p.B <= ctx->tc_bn_max &&
+    // decode batches above 128 keep the fp32 products of the CUDA-core GEMV;
+    // prefill chunks may be as tall as their buffers
+    const int most = ctx->rows > ctx->B ? ctx->tc_bn_max : std::min(ctx->tc_bn_max, 128);
+    return ctx->cfg.dtype == 1 && ctx->tc_xb && p.B >= ctx->tc_min_b && p.B <= most &&
            p.K % kTcBK == 0 && p.K <= ctx->tc_kmax && p.K <= 4 * kPrepQ * kPrepThreads && rows >= kTcM;
 }
 
@@ -831,6 +932,7 @@ cudaError_t set_carveouts(bool bf) {
         for (int bn : {16, 32, 64, 128})
             for (bool deep : {false, true})
                 for (bool fused : {false, true}) fns.push_back(pick_tcv(bn, deep, fused));
+        for (int nt : {128, kPairMaxN}) fns.push_back(k_pick_pair(nt));
         fns.push_back(reinterpret_cast<const void*>(k_pick_prep_bf16()));
         for (int g : {1, 2, 4})
             for (bool deep : {false, true}) fns.push_back(attnm_pick(g, deep));
@@ -1678,14 +1780,14 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         // activations and state
         const int qd = c.n_q_heads * DH, kd = c.n_kv_heads * DH;
         // prefill chunks: PIPO_PREFILL_ROWS=<rows> (positions x sequences per
-        // chunk, at most 128; 0 or unset: one position at a time)
-        if (const char* ev = getenv("PIPO_PREFILL_ROWS")) ctx->prefill_rows = std::min(128, std::max(0, atoi(ev)));
+        // chunk, at most kMaxPrefillRows; 0 or unset: one position at a time)
+        if (const char* ev = getenv("PIPO_PREFILL_ROWS")) ctx->prefill_rows = std::min(kMaxPrefillRows, std::max(0, atoi(ev)));
         if (const char* ev = getenv("PIPO_PREFILL_ATTN")) ctx->prefill_tile_attn = strcmp(ev, "tile") == 0;
         const int MR = std::max(MB, ctx->prefill_rows);
         ctx->max_rows = MR;
         // GEMM inputs get at least as many rows as the tensor-core batch width
         // (their activation tensor maps read box-sized tiles of BH rows)
-        ctx->act_rows = c.dtype == 1 ? std::max(MR, tc_bn(std::min(MR, 128))) : MR;
+        ctx->act_rows = c.dtype == 1 ? std::max(MR, tc_bn(MR)) : MR;
         const size_t AR = (size_t)ctx->act_rows;
         TRY(dalloc(ctx, &ctx->x, AR * H * 4));
         TRY(dalloc(ctx, &ctx->x2, AR * H * 4));
@@ -1708,7 +1810,7 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         if (const char* ev = getenv("PIPO_ATTN_MMA_MIN_BATCH")) ctx->attn_mma_min_b = std::max(1, atoi(ev));
         if (const char* ev = getenv("PIPO_TC_SPLITS")) ctx->tc_splits = std::max(0, atoi(ev));
         if (c.dtype == 1 && MR >= ctx->tc_min_b) {
-            ctx->tc_bn_max = tc_bn(std::min(MR, 128));
+            ctx->tc_bn_max = tc_bn(std::max(std::min(MB, 128), ctx->prefill_rows));
             ctx->tc_kmax = std::max({2 * (int)H, qd, c.ffn});
             TRY(dalloc(ctx, &ctx->tc_xb, (size_t)2 * ctx->tc_bn_max * ctx->tc_kmax * 2));
         }
