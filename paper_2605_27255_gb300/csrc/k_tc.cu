@@ -42,10 +42,7 @@ void* k_pick_tcv(int bh, bool deep, bool fused) {
     return deep ? pick_tc_v<true>(bh) : pick_tc_v<false>(bh);
 }
 
-void* k_pick_pair(int nt) {
-    return nt <= 128 ? reinterpret_cast<void*>(&gemm_pair_kernel<128>)
-                     : reinterpret_cast<void*>(&gemm_pair_kernel<kPairMaxN>);
-}
+void* k_pick_pair() { return reinterpret_cast<void*>(&gemm_pair_kernel<kPairN>); }
 
 void* k_pick_prep_bf16() { return reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16>); }
 

@@ -296,7 +296,6 @@ constexpr size_t kXsBudget = 100 * 1024;      // fp32 bytes of the longest GEMV 
 // cached keys and values); longer slices take the register ring alone
 constexpr size_t kAttnStageMax = 160 * 1024;
 constexpr int kMaxPrefillRows = 2048;         // rows of a prefill chunk (PIPO_PREFILL_ROWS)
-constexpr size_t kPairSmemMax = 208 * 1024;   // stages of the CTA-pair GEMM (one CTA per SM)
 constexpr size_t kBlkSmemMax = (size_t)kBlkKMax * kBlkNB * 4 + (size_t)kBlkSeg * 32 * 4;
 constexpr size_t kStreamBudget = 200 * 1024;  // staged-input bytes per streaming GEMV block
 
@@ -428,11 +427,7 @@ cudaError_t set_smem_attrs(bool bf) {
                                                                  : cudaClusterSchedulingPolicyLoadBalancing);
                     if (e != cudaSuccess) return e;
                 }
-    if (bf)
-        for (int nt : {128, kPairMaxN}) {
-            cudaError_t e = cudaFuncSetAttribute(k_pick_pair(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemMax);
-            if (e != cudaSuccess) return e;
-        }
+    if (bf) return cudaFuncSetAttribute(k_pick_pair(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
     return cudaSuccess;
 }
 
@@ -485,6 +480,23 @@ pipo_status make_tmap_x(pipo_ctx* ctx, CUtensorMap* tm, const float* base, int K
                                       box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(ctx, PIPO_ECUDA, "cuTensorMapEncodeTiled (activations): error %d", (int)r);
+    return PIPO_OK;
+}
+
+// 2-D fp32 tensor map of outputs [rows][ld] (first N columns) for stores of
+// boxes of box_n columns x box_rows rows.
+pipo_status make_tmap_y(pipo_ctx* ctx, CUtensorMap* tm, float* base, int N, int ld, int rows, int box_n, int box_rows) {
+    TRY(load_encoder(ctx));
+    if (!base || reinterpret_cast<uintptr_t>(base) % 16 != 0 || ld % 4 != 0 || N < 1 || rows < 1)
+        return fail(ctx, PIPO_EINVAL, "output tensor map: base %% 16, ld %% 4 required");
+    const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
+    const cuuint32_t box[2] = {(cuuint32_t)box_n, (cuuint32_t)box_rows};
+    const cuuint32_t es[2] = {1, 1};
+    const CUresult r = g_encode_tiled(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, es,
+                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, PIPO_ECUDA, "cuTensorMapEncodeTiled (outputs): error %d", (int)r);
     return PIPO_OK;
 }
 
@@ -613,19 +625,18 @@ int tc_fused_max_bh() {
 
 // CTA pairs of the CTA-pair GEMM that can be resident at once on the current
 // device (cached).
-int pair_max_clusters(int nt, size_t smem) {
+int pair_max_clusters() {
     static std::mutex mu;
-    static std::map<long long, int> cache;
+    static std::map<int, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
-    const long long key = ((long long)dev << 40) | ((long long)(nt <= 128) << 32) | (long long)smem;
     std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(key);
+    auto it = cache.find(dev);
     if (it != cache.end()) return it->second;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(2);
     lc.blockDim = dim3(kPairThreads);
-    lc.dynamicSmemBytes = smem;
+    lc.dynamicSmemBytes = kPairSmem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
@@ -634,38 +645,12 @@ int pair_max_clusters(int nt, size_t smem) {
     lc.attrs = at;
     lc.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_pick_pair(nt), &lc) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_pick_pair(), &lc) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
     }
-    cache[key] = n;
+    cache[dev] = n;
     return n;
-}
-
-// Launch plan of the CTA-pair GEMM: positions per tile, stages, pairs.  The R
-// positions are cut into equal tiles whose width makes the persistent pairs'
-// rounds shortest in total.  A 64-wide K block of a tile takes 4 NT
-// tensor-core clocks, and the 16 KB + 128 NT bytes a CTA loads for it arrive
-// at about 48 bytes per clock: 2.7 (NT + 128) clocks, the larger of the two up
-// to NT = 256.
-struct PairPlan {
-    int NT, ST, pairs;
-    size_t smem;
-};
-PairPlan pair_plan(int sms, int rows, int R) {
-    const int mt = (rows + kPairM - 1) / kPairM, pairs = std::max(1, sms / 2);
-    PairPlan pl{};
-    long long best = -1;
-    for (int nt = 32; nt <= kPairMaxN; nt += 32) {
-        const long long tiles = (long long)mt * ((R + nt - 1) / nt), cost = (tiles + pairs - 1) / pairs * (nt + 128);
-        if (best < 0 || cost <= best) { best = cost; pl.NT = nt; }
-    }
-    pl.ST = kPairMaxStages;
-    while (pl.ST > 2 && pair_smem(pl.NT, pl.ST) > kPairSmemMax) --pl.ST;
-    pl.smem = pair_smem(pl.NT, pl.ST);
-    const int tiles = mt * ((R + pl.NT - 1) / pl.NT);
-    pl.pairs = std::min(tiles, std::max(1, pair_max_clusters(pl.NT, pl.smem)));
-    return pl;
 }
 
 // Projection of a prefill chunk of more than 128 rows: bf16 hi and lo rows
@@ -673,17 +658,15 @@ PairPlan pair_plan(int sms, int rows, int R) {
 pipo_status launch_gemm_pair(pipo_ctx* ctx, const GemvParams& p, bf16* xb) {
     if (p.epi == EPI_ARGMAX) return fail(ctx, PIPO_EINVAL, "argmax of %d rows on the CTA-pair GEMM", p.B);
     const int ru = p.epi == EPI_SWIGLU ? 2 : 1, rows = p.N * ru;
-    const PairPlan pl = pair_plan(ctx->sms, rows, p.B);
     PairParams q{};
-    q.t.rows = rows; q.t.K = p.K; q.t.B = p.B; q.t.ru = ru; q.t.epi = p.epi;
-    q.t.y = p.y; q.t.ldy = p.ldy; q.t.bias = p.bias;
-    q.NT = pl.NT;
-    q.ST = pl.ST;
-    q.tiles_n = (p.B + pl.NT - 1) / pl.NT;
+    q.rows = rows; q.K = p.K; q.B = p.B; q.ru = ru; q.epi = p.epi; q.bias = p.bias;
+    q.tiles_n = (p.B + kPairN - 1) / kPairN;
     q.tiles = (rows + kPairM - 1) / kPairM * q.tiles_n;
-    CUtensorMap tmW, tmX;
+    const int pairs = std::min(q.tiles, std::max(1, pair_max_clusters()));
+    CUtensorMap tmW, tmX, tmY;
     TRY(make_tmap(ctx, &tmW, p.W, p.K, rows, kTcM));
-    TRY(make_tmap(ctx, &tmX, xb, p.K, 2 * p.B, pl.NT / 2));
+    TRY(make_tmap(ctx, &tmX, xb, p.K, 2 * p.B, kPairN / 2));
+    TRY(make_tmap_y(ctx, &tmY, p.y, p.N, p.ldy, p.B, 32 / ru, kPairOutN));
     {
         GemvParams pp = p;
         int bh = p.B;
@@ -693,10 +676,10 @@ pipo_status launch_gemm_pair(pipo_ctx* ctx, const GemvParams& p, bf16* xb) {
         ctx->launch_prep = true;
         TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16()), dim3(p.B), dim3(kPrepThreads), 0, args));
     }
-    void* args[] = {&tmW, &tmX, &q};
+    void* args[] = {&tmW, &tmX, &tmY, &q};
     ctx->prof_kind = 0;
     ctx->prof_bytes = (double)rows * p.K * 2;
-    return launch_ex(ctx, k_pick_pair(pl.NT), dim3(2 * pl.pairs), dim3(kPairThreads), pl.smem, args, 2);
+    return launch_ex(ctx, k_pick_pair(), dim3(2 * pairs), dim3(kPairThreads), kPairSmem, args, 2);
 }
 
 // Projection on the tensor cores: the fused GEMM, or bf16 activations from
@@ -932,7 +915,7 @@ cudaError_t set_carveouts(bool bf) {
         for (int bn : {16, 32, 64, 128})
             for (bool deep : {false, true})
                 for (bool fused : {false, true}) fns.push_back(pick_tcv(bn, deep, fused));
-        for (int nt : {128, kPairMaxN}) fns.push_back(k_pick_pair(nt));
+        fns.push_back(k_pick_pair());
         fns.push_back(reinterpret_cast<const void*>(k_pick_prep_bf16()));
         for (int g : {1, 2, 4})
             for (bool deep : {false, true}) fns.push_back(attnm_pick(g, deep));
@@ -1529,12 +1512,42 @@ pipo_status enqueue_prefill_chunk(pipo_ctx* ctx, bool regular, int j0, int C) {
     return launch_ex(ctx, (const void*)&advance_kernel, dim3((B + 127) / 128), dim3(128), 0, args);
 }
 
+// Rows of a chunk: as many as the caller allows, unless fewer fill the
+// CTA-pair GEMM's rounds better.  The tiles of a block's projections (256
+// outputs x 256 rows) go round the resident pairs, a round of a projection
+// taking time with its K whether its last one is full or not: at the 4B
+// shapes 2048 rows are 80 tiles of O and of the down projection on 76 pairs,
+// two rounds, and 1792 rows 70 tiles, one.  Chosen: the n * 256 rows of the
+// least rounds x K per row, a chunk's launches standing for kChunkK inputs
+// (about 40 us per block at 0.6 us per 64 inputs of a round).
+constexpr int kChunkK = 4300;
+int prefill_chunk_rows(const pipo_ctx* ctx) {
+    const pipo_config& c = ctx->cfg;
+    if (ctx->prefill_rows < 2 * kPairN || c.dtype != 1) return ctx->prefill_rows;
+    const int pairs = std::max(1, pair_max_clusters()), qd = c.n_q_heads * c.head_dim, kd = c.n_kv_heads * c.head_dim;
+    const int shp[4][2] = {{qd + 2 * kd, c.hidden}, {c.hidden, qd}, {2 * c.ffn, c.hidden}, {c.hidden, c.ffn}};
+    int best = ctx->prefill_rows;
+    double best_cost = -1.0;
+    for (int n = ctx->prefill_rows / kPairN; n >= 1; --n) {
+        double k = kChunkK;
+        for (auto& s : shp) {
+            const long long tiles = (long long)((s[0] + kPairM - 1) / kPairM) * n;
+            k += (double)((tiles + pairs - 1) / pairs) * s[1];
+        }
+        if (best_cost < 0.0 || k / n < best_cost) {
+            best_cost = k / n;
+            best = n * kPairN;
+        }
+    }
+    return best;
+}
+
 // The positions before a prompt's last one in chunks of prefill_rows / B
 // positions (when chunks are enabled and hold two or more positions);
 // *j receives the first position left for the position-by-position path.
 pipo_status enqueue_prefill_chunks(pipo_ctx* ctx, bool regular, int N, int* j) {
     const int B = ctx->B;
-    const int cmax = ctx->prefill_rows / B;
+    const int cmax = prefill_chunk_rows(ctx) / B;
     *j = 0;
     if (cmax < 2 || ctx->attn_v0) return PIPO_OK;
     while (N - 1 - *j >= 2) {

@@ -14,7 +14,8 @@
 // error of the SwiGLU outputs, 4.4e-6 with the K splits of the narrow kernels).
 // Every kPairSeg K blocks the accumulator is therefore handed to the epilogue
 // warps, which add it to fp32 sums in their registers (rounding to nearest)
-// while the MMAs go on in the other TMEM buffer: @PREC@
+// while the MMAs go on in the other TMEM buffer: 3.6e-6, and 2.5e-6 at K = 9728
+// (the narrow kernels 2.7e-6).
 //
 // Roles per CTA: warp 0 issues its CTA's TMA copies, which complete on the
 // leader's (even rank) barrier; one thread of the leader issues the MMAs for
@@ -23,7 +24,14 @@
 // pair c takes tiles c, c + pairs, ...; a tile's outputs are written while the
 // next tile's MMAs run.  Every wait is bounded (error word; the other roles
 // give up the same way).
-// @PERF@
+//
+// Measured at R = 2048 and the 4B shapes (TFLOP/s of hi and lo products, of a
+// dense bf16 fallback peak of 1900): QKV 1422, gate/up 1583, down 992 (80 tiles
+// on 76 pairs: the chunk planner avoids such heights).  Without the epilogue
+// the loop runs at 2100: the rest is TMEM reads and the output phase, during
+// which the MMAs are at most two segments ahead.  A position tile narrower
+// than 256 saves nothing: the 8 MMAs of a K block take about 1050 clocks at
+// any width (the weight operand bounds them).
 #pragma once
 
 #include "tcgen05_gemm.cuh"
@@ -35,23 +43,25 @@ constexpr int kPairEpiWarps = 8;
 constexpr int kPairThreads = 128 + 32 * kPairEpiWarps;  // warpgroup 0: copies, MMAs (two warps idle)
 // registers: 3 warpgroups are launched with 168 a thread; the two epilogue
 // warpgroups hold 128 sums a thread and take what warpgroup 0 gives back
-// (72 + 2 * 216 = 3 * 168)
-constexpr int kPairRegsIo = 72, kPairRegsEpi = 216;
+// (56 + 2 * 224 = 3 * 168)
+constexpr int kPairRegsIo = 56, kPairRegsEpi = 224;
 static_assert(kPairRegsIo + 2 * kPairRegsEpi <= 3 * 168, "register shares must fit the launch's registers");
-constexpr int kPairMaxN = 256;       // positions per tile (a multiple of 32)
-constexpr int kPairMaxStages = 8;
+constexpr int kPairN = 256;          // positions per tile
+constexpr int kPairStages = 4;
+constexpr int kPairOutN = 16;        // positions per output store of a warp
 constexpr int kPairSeg = 4;          // 64-wide K blocks per accumulator segment
 
-__host__ __device__ constexpr int pair_stage_bytes(int nt) { return kTcABytes + nt * 128; }
-__host__ __device__ constexpr size_t pair_smem(int nt, int st) {
-    return 1024 + (size_t)st * pair_stage_bytes(nt) + (2 * st + 4) * 8;
-}
+constexpr int kPairStageBytes = kTcABytes + kPairN * 128;  // weights, half of the hi and of the lo rows
+constexpr size_t kPairSmem =
+    1024 + (size_t)kPairStages * kPairStageBytes + kPairEpiWarps * 2 * kPairOutN * 32 * 4 + (2 * kPairStages + 4) * 8;
 
 struct PairParams {
-    TcParams t;      // rows, K, B = positions, ru, epi, outputs (splits: unused)
-    int NT, ST;      // positions per tile, stages
-    int tiles_n;     // position tiles
-    int tiles;       // weight tiles * position tiles
+    int rows;          // W rows (outputs * ru)
+    int K, B;          // inputs, positions
+    int ru, epi;       // as TcParams
+    const void* bias;  // bf16 [rows]
+    int tiles_n;       // position tiles
+    int tiles;         // weight tiles * position tiles
 };
 
 // shared::cluster address of a local shared address in the CTA of rank `rank`
@@ -90,7 +100,9 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint16_t mask) {
 }
 
 __device__ __forceinline__ void mbar_arrive_at(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    // CTA-scope release: what it orders are TMEM reads (tcgen05 fence); a
+    // cluster-scope one would wait for the tile's global stores
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -102,50 +114,59 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Outputs of weight row `row` (one per lane; the warp's 32 rows are
-// consecutive) and positions [b0, b1), b1 <= b0 + 16, with sums v.
-__device__ __forceinline__ void pair_epilogue(const TcParams& p, int row, int b0, int b1, const float* v) {
-    const bool in = row < p.rows;
-    if (p.ru == 2) {  // gate on even rows, up on the odd row after it
+// shared -> global 2-D tensor store (or fp32 add) of the box at element
+// coordinates (x, y); parts outside the tensor are left out
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, int x, int y, const void* src, bool add) {
+    if (add)
+        asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tm),
+                     "r"(x), "r"(y), "r"(smem_u32(src))
+                     : "memory");
+    else
+        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tm), "r"(x),
+                     "r"(y), "r"(smem_u32(src))
+                     : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// 64 consecutive fp32 columns of this thread's TMEM lane, one wait
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
+    uint32_t r[64];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const float up = __shfl_xor_sync(0xffffffffu, v[j], 1);
-            if (in && (row & 1) == 0 && b0 + j < b1) p.y[(size_t)(b0 + j) * p.ldy + (row >> 1)] = silu(v[j]) * up;
-        }
-        return;
-    }
-    if (!in) return;
-    float* yp = p.y + (size_t)b0 * p.ldy + row;
-    if (p.epi == EPI_RESADD) {
-        float r[16];
+    for (int h = 0; h < 2; ++h)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,"
+            "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+            : "=r"(r[32 * h + 0]), "=r"(r[32 * h + 1]), "=r"(r[32 * h + 2]), "=r"(r[32 * h + 3]),
+              "=r"(r[32 * h + 4]), "=r"(r[32 * h + 5]), "=r"(r[32 * h + 6]), "=r"(r[32 * h + 7]),
+              "=r"(r[32 * h + 8]), "=r"(r[32 * h + 9]), "=r"(r[32 * h + 10]), "=r"(r[32 * h + 11]),
+              "=r"(r[32 * h + 12]), "=r"(r[32 * h + 13]), "=r"(r[32 * h + 14]), "=r"(r[32 * h + 15]),
+              "=r"(r[32 * h + 16]), "=r"(r[32 * h + 17]), "=r"(r[32 * h + 18]), "=r"(r[32 * h + 19]),
+              "=r"(r[32 * h + 20]), "=r"(r[32 * h + 21]), "=r"(r[32 * h + 22]), "=r"(r[32 * h + 23]),
+              "=r"(r[32 * h + 24]), "=r"(r[32 * h + 25]), "=r"(r[32 * h + 26]), "=r"(r[32 * h + 27]),
+              "=r"(r[32 * h + 28]), "=r"(r[32 * h + 29]), "=r"(r[32 * h + 30]), "=r"(r[32 * h + 31])
+            : "r"(taddr + 32 * h));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    // the values exist from here on: nothing may use them before the wait
 #pragma unroll
-        for (int j = 0; j < 16; ++j) r[j] = b0 + j < b1 ? __ldcg(yp + (size_t)j * p.ldy) : 0.f;
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (b0 + j < b1) yp[(size_t)j * p.ldy] = r[j] + v[j];
-        return;
-    }
-    const float bias = p.epi == EPI_BIAS ? __bfloat162float(static_cast<const __nv_bfloat16*>(p.bias)[row]) : 0.f;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float a = v[j];
-        if (p.epi == EPI_BIAS) a += bias;
-        else if (p.epi == EPI_SILU) a = silu(a);
-        if (b0 + j < b1) yp[(size_t)j * p.ldy] = a;
+    for (int i = 0; i < 64; ++i) {
+        asm volatile("" : "+r"(r[i]));
+        v[i] = __uint_as_float(r[i]);
     }
 }
 
 // clusters of two CTAs; tmW boxes 64 x 128 rows, tmX boxes 64 x NT / 2 rows of
-// the [2R][K] operand; NT <= MAXN
-template <int MAXN>
+// the [2R][K] operand, tmY boxes of a warp's 32 / ru outputs x kPairOutN positions
+template <int NT>
 __global__ void __launch_bounds__(kPairThreads, 1)
-    gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, PairParams q) {
+    gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
+                     const __grid_constant__ CUtensorMap tmY, PairParams p) {
     extern __shared__ __align__(1024) unsigned char tp_smem_raw[];
     __shared__ uint32_t tmem_base;
-    const TcParams& p = q.t;
-    const int NT = q.NT, ST = q.ST, SB = pair_stage_bytes(NT);
+    constexpr int ST = kPairStages, SB = kPairStageBytes;
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tp_smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t* full = reinterpret_cast<uint64_t*>(sm + (size_t)ST * SB);  // leader's: both CTAs' copies of a stage
+    float* out_s = reinterpret_cast<float*>(sm + (size_t)ST * SB);  // [epilogue warps][2][kPairOutN][32]
+    uint64_t* full = reinterpret_cast<uint64_t*>(out_s + kPairEpiWarps * 2 * kPairOutN * 32);  // leader's: both CTAs'
+                                                                                            // copies of a stage
     uint64_t* empty = full + ST;   // this CTA's: the MMAs have read the stage
     uint64_t* accf = empty + ST;   // [2] this CTA's: a segment's sums are in the buffer
     uint64_t* acce = accf + 2;     // [2] leader's: buffer read by the epilogue warps of both CTAs
@@ -155,12 +176,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     const int half = (int)rank;
     const int cid = (int)blockIdx.x / 2, ncl = (int)gridDim.x / 2;
     const int nk = p.K / kTcBK;
-    uint32_t cols = 32;        // TMEM columns: two buffers of NT
-    while ((int)cols < 2 * NT) cols <<= 1;
+    constexpr uint32_t cols = 2 * NT;  // TMEM columns: two buffers (all of an SM's)
+    static_assert(NT == 256, "the epilogue warps' shares and the TMEM buffers");
 
     if (threadIdx.x == 64) {
         prefetch_tmap(&tmW);
         prefetch_tmap(&tmX);
+        prefetch_tmap(&tmY);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
@@ -206,8 +228,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                 };
                 int it = 0;
                 bool ok = true;
-                for (int t = cid; t < q.tiles && ok; t += ncl) {
-                    const int m = t / q.tiles_n, n = t % q.tiles_n;
+                for (int t = cid; t < p.tiles && ok; t += ncl) {
+                    const int m = t / p.tiles_n, n = t % p.tiles_n;
                     int i = 0;
                     if (t == cid) {
                         // the first stages' weights need nothing from the kernel before
@@ -237,7 +259,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                 const uint32_t idesc = umma_idesc_bf16(kPairM, NT);
                 int it = 0, sc = 0;
                 bool ok = true;
-                for (int t = cid; t < q.tiles && ok; t += ncl) {
+                for (int t = cid; t < p.tiles && ok; t += ncl) {
                     for (int i0 = 0; i0 < nk && ok; i0 += kPairSeg, ++sc) {
                         const int buf = sc & 1, i1 = min(nk, i0 + kPairSeg);
                         if (sc >= 2 && !mbar_wait(acce + buf, (uint32_t)(((sc >> 1) & 1) ^ 1), 33, sc)) { ok = false; break; }
@@ -267,38 +289,78 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kPairRegsEpi));
         // ---- epilogue: warps w own TMEM lane quadrant w % 4 and the positions
         // [ch, ch + NT / 2) of the tile
-        const int quad = warp & 3, nc = NT / 2, ch = (warp - 4) / 4 * nc;
+        constexpr int nc = NT / 2;
+        const int quad = warp & 3, ch = (warp - 4) / 4 * nc;
         const uint32_t acce_lead = map_rank(smem_u32(acce), 0);
         const uint32_t src = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)ch;
+        float* mine = out_s + (warp - 4) * 2 * kPairOutN * 32;
         pdl_wait();
-        int sc = 0;
+        int sc = 0, oc = 0;  // segments, output stores so far
         bool ok = true;
-        for (int t = cid; t < q.tiles && ok; t += ncl) {
-            const int m = t / q.tiles_n, n = t % q.tiles_n;
-            float acc[MAXN / 2];
+        for (int t = cid; t < p.tiles && ok; t += ncl) {
+            const int m = t / p.tiles_n, n = t % p.tiles_n;
+            float acc[nc];
+#pragma unroll
+            for (int j = 0; j < nc; ++j) acc[j] = 0.f;
             for (int i0 = 0; i0 < nk; i0 += kPairSeg, ++sc) {
                 const int buf = sc & 1;
                 if (!mbar_wait(accf + buf, (uint32_t)((sc >> 1) & 1), 35, sc)) { ok = false; break; }
                 __syncwarp();
                 tc_fence_after();
+                // 64 columns per wait: with 16 the loads' latency, eight times
+                // per segment, held the MMAs up (gate/up 290 us, 258 with 64)
 #pragma unroll
-                for (int c0 = 0; c0 < MAXN / 2; c0 += 16)
-                    if (c0 < nc) {
-                        float v[16];
-                        tmem_ld16(src + (uint32_t)(buf * NT + c0), v);
+                for (int c0 = 0; c0 < nc; c0 += 64) {
+                    float v[64];
+                    tmem_ld64(src + (uint32_t)(buf * NT + c0), v);
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) acc[c0 + j] = i0 == 0 ? v[j] : acc[c0 + j] + v[j];
-                    }
+                    for (int j = 0; j < 64; ++j) acc[c0 + j] += v[j];
+                }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(acce_lead + 8 * buf);
             }
             if (!ok) break;
-            const int row = m * kPairM + half * 128 + quad * 32 + lane, b0 = n * NT + ch, bmax = min(p.B, b0 + nc);
+            // outputs through the warp's two buffers [kPairOutN][32 / ru] and
+            // tensor stores, which overlap the next tile (its MMAs wait for
+            // these warps after two segments)
+            const int b0 = n * NT + ch, ru = p.ru, row0 = m * kPairM + half * 128 + quad * 32, row = row0 + lane;
+            const float bias = p.epi == EPI_BIAS && row < p.rows
+                                   ? __bfloat162float(static_cast<const __nv_bfloat16*>(p.bias)[row]) : 0.f;
 #pragma unroll
-            for (int c0 = 0; c0 < MAXN / 2; c0 += 16)
-                if (c0 < nc) pair_epilogue(p, row, b0 + c0, bmax, acc + c0);
+            for (int c0 = 0; c0 < nc; c0 += kPairOutN)
+                if (b0 + c0 < p.B && row0 < p.rows) {
+                    float* buf = mine + (oc++ & 1) * kPairOutN * 32;
+                    // the store issued from this buffer before last has read it
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    __syncwarp();
+                    if (ru == 2) {
+                        // gate on even rows, up on the odd row after it: of every
+                        // two positions the even lane finishes the first, the odd
+                        // lane the second
+                        const bool odd = lane & 1;
+#pragma unroll
+                        for (int j = 0; j < kPairOutN; j += 2) {
+                            const float v0 = acc[c0 + j], v1 = acc[c0 + j + 1];
+                            const float o = __shfl_xor_sync(0xffffffffu, odd ? v0 : v1, 1);
+                            buf[(j + odd) * 16 + (lane >> 1)] = silu(odd ? o : v0) * (odd ? v1 : o);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < kPairOutN; ++j) {
+                            float a = acc[c0 + j];
+                            if (p.epi == EPI_BIAS) a += bias;
+                            else if (p.epi == EPI_SILU) a = silu(a);
+                            buf[j * 32 + lane] = a;
+                        }
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    // EPI_RESADD: every output has one writer, the add at L2 is y + v rounded once
+                    if (lane == 0) tma_store_2d(&tmY, row0 / ru, b0 + c0, buf, p.epi == EPI_RESADD);
+                }
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         __syncwarp();
     }
     tc_fence_before();
