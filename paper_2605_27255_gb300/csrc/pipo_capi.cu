@@ -140,7 +140,8 @@ struct pipo_ctx {
     size_t multi_cap = 0;
 
     float* rope = nullptr;            // [max_ctx][d_h/2][2] cos, sin
-    bool pdl = false;                 // programmatic dependent launch (decode graph only)
+    bool pdl = false;                 // programmatic dependent launch (decode graph, prefill)
+    bool pdl_eager = false;           // ... of launches outside a graph: the attention waits for the launch before
     bool attn_cs16 = false;           // 16-CTA attention clusters available
     int attn_cs_force = 0;            // (development) fixed attention cluster size
     int attn_cs_target = 0;           // attention CTAs per SM above which clusters shrink (0: per kernel)
@@ -174,7 +175,7 @@ struct pipo_ctx {
     int rows = 0;                     // activation rows of the enqueue in progress (0: B, one per sequence)
     int max_rows = 0;                 // rows the activation buffers hold: max(max_batch, prefill_rows)
     int prefill_rows = 0;             // rows of a prefill chunk (positions x sequences; 0: one position at a time)
-    bool prefill_tile_attn = false;   // chunk attention by tiles of positions (attn_prefill_kernel)
+    int prefill_attn = 0;             // chunk attention: 0 by size, 1 row by row, 2 causal tiles (attn_prefill_kernel)
     // sampling in both heads (pipo_set_sampler; greedy when off)
     bool samp_on = false;
     float samp_T = 1.f, samp_p = 1.f, samp_rep = 1.f;
@@ -1116,6 +1117,18 @@ size_t attn_stage(const pipo_ctx* ctx, int splits, bool chunk, int* stage_max) {
     return bytes;
 }
 
+// Attention of a prefill chunk of R rows by causal tiles: PIPO_PREFILL_ATTN,
+// or else from 64 rows and 8 positions per sequence on.  Measured (prompt of
+// two 4B-wide layers, ms, row by row / tiles): 8000 tokens of one sequence 32
+// rows 59.6 / 63.2, 64 rows 45.2 / 36.7, 128 rows 37.1 / 23.0; 4 x 2000 tokens
+// 32 rows 45.0 / 48.3, 64 rows 30.8 / 29.8; 16 x 400 tokens 64 rows (4 positions)
+// 21.7 / 22.5, 128 rows 15.3 / 15.0.
+bool prefill_tiles(const pipo_ctx* ctx, int R) {
+    if (!attn_mma_ok(ctx) || (int)ctx->kv_tm.size() != 2 * ctx->n_cache_layers) return false;
+    if (ctx->prefill_attn > 0) return ctx->prefill_attn == 2;
+    return R >= 64 && R / ctx->B >= 8;
+}
+
 // One decoder block on the residual stream xr (pre-norm attention + SwiGLU).
 pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, float* xr) {
     const pipo_config& c = ctx->cfg;
@@ -1126,7 +1139,7 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
     p.seg[0] = act_seg(xr, H, H, bw.attn_norm);
     p.K = H;
     KVView kv = kv_view(ctx, cache_layer);
-    if (attn_l2_warm() && (ctx->rows <= 0 || ctx->rows == ctx->B)) {
+    if (attn_l2_warm() && !ctx->pdl_eager && (ctx->rows <= 0 || ctx->rows == ctx->B)) {
         // a decode step: the streaming GEMV warms L2 with this layer's cached pages
         p.pf_k = kv.K;
         p.pf_v = kv.V;
@@ -1153,6 +1166,14 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
             void* fn = k_pick_append_rows(bf, DH);
             TRY(launch_ex(ctx, fn, dim3(R, c.n_kv_heads), dim3(DH / 2), 0, args));
         }
+        // outside a graph a launch or two earlier may still write the lengths
+        // and entries that the attention reads before its dependency wait
+        struct PdlGuard {
+            pipo_ctx* c;
+            bool was;
+            ~PdlGuard() { c->pdl = was; }
+        } guard{ctx, ctx->pdl};
+        if (ctx->pdl_eager && !(chunk && prefill_tiles(ctx, R))) ctx->pdl = false;
         ctx->prof_kind = 1;
         ctx->prof_bytes = 0.0;
         for (int b = 0; b < ctx->B && b < (int)ctx->h_len.size(); ++b)
@@ -1170,7 +1191,7 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
         void* args[] = {&ap};
         const int cs = attn_cluster_size(ctx, R);
         const int G = c.n_q_heads / c.n_kv_heads;
-        if (chunk && ctx->prefill_tile_attn && attn_mma_ok(ctx) && (int)ctx->kv_tm.size() == 2 * ctx->n_cache_layers) {
+        if (chunk && prefill_tiles(ctx, R)) {
             // causal tiles: the positions of a tile share every key and value they read
             void* fn = k_pick_attn_prefill(G);
             CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prefill_attn_smem()));
@@ -1311,6 +1332,15 @@ pipo_status enqueue_sample(pipo_ctx* ctx, const float* logits, int head, unsigne
     void* args[] = {&sp};
     return launch_ex(ctx, (const void*)&sample_kernel, dim3(samp_slices(c.vocab), ctx->B), dim3(kSampThreads), 0, args);
 }
+
+// Launches of a prefill in one stream: every kernel reads only weights and
+// gains before its dependency wait (the attention aside, see enqueue_block), and
+// a kernel that has ended has waited for the one before it.
+struct EagerPdl {
+    pipo_ctx* c;
+    explicit EagerPdl(pipo_ctx* ctx) : c(ctx) { c->pdl = c->pdl_eager = true; }
+    ~EagerPdl() { c->pdl = c->pdl_eager = false; }
+};
 
 // One pair position of every sequence.  DECODE: the pending pair; PREFILL_*:
 // prompt pair j.  PREFILL_MID stops after the MTP block (teacher-forced token).
@@ -1795,7 +1825,7 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         // prefill chunks: PIPO_PREFILL_ROWS=<rows> (positions x sequences per
         // chunk, at most kMaxPrefillRows; 0 or unset: one position at a time)
         if (const char* ev = getenv("PIPO_PREFILL_ROWS")) ctx->prefill_rows = std::min(kMaxPrefillRows, std::max(0, atoi(ev)));
-        if (const char* ev = getenv("PIPO_PREFILL_ATTN")) ctx->prefill_tile_attn = strcmp(ev, "tile") == 0;
+        if (const char* ev = getenv("PIPO_PREFILL_ATTN")) ctx->prefill_attn = strcmp(ev, "tile") == 0 ? 2 : 1;
         const int MR = std::max(MB, ctx->prefill_rows);
         ctx->max_rows = MR;
         // GEMM inputs get at least as many rows as the tensor-core batch width
@@ -2048,10 +2078,13 @@ pipo_status pipo_prefill(pipo_ctx* ctx, int32_t batch, const int32_t* h_ids, int
     ctx->h_len.assign(batch, 0);
     const int saved = ctx->launches;
     int j = 0;
-    TRY(enqueue_prefill_chunks(ctx, false, N, &j));
-    for (; j < N; ++j) {
-        TRY(enqueue_position(ctx, j + 1 < N ? PREFILL_MID : PREFILL_LAST, j));
-        ctx->h_len.assign(batch, j + 1);
+    {
+        EagerPdl eager(ctx);
+        TRY(enqueue_prefill_chunks(ctx, false, N, &j));
+        for (; j < N; ++j) {
+            TRY(enqueue_position(ctx, j + 1 < N ? PREFILL_MID : PREFILL_LAST, j));
+            ctx->h_len.assign(batch, j + 1);
+        }
     }
     ctx->launches = saved;
     if (h_tokens) CK(cudaMemcpyAsync(h_tokens, ctx->out_tokens, (size_t)batch * 8, cudaMemcpyDeviceToHost, ctx->stream));
@@ -2156,10 +2189,13 @@ pipo_status pipo_regular_prefill(pipo_ctx* ctx, int32_t batch, const int32_t* h_
     ctx->h_len.assign(batch, 0);
     const int saved = ctx->launches;
     int j = 0;
-    TRY(enqueue_prefill_chunks(ctx, true, N, &j));
-    for (; j < N; ++j) {
-        TRY(enqueue_regular(ctx, j + 1 < N ? PREFILL_MID : PREFILL_LAST, j));
-        ctx->h_len.assign(batch, j + 1);
+    {
+        EagerPdl eager(ctx);
+        TRY(enqueue_prefill_chunks(ctx, true, N, &j));
+        for (; j < N; ++j) {
+            TRY(enqueue_regular(ctx, j + 1 < N ? PREFILL_MID : PREFILL_LAST, j));
+            ctx->h_len.assign(batch, j + 1);
+        }
     }
     ctx->launches = saved;
     // the prefill's token is the first output, not a decode step's
@@ -2737,7 +2773,7 @@ pipo_status pipo_describe_step(const pipo_ctx* ctx, char* h_buf, size_t cap) {
     d += ctx->samp_on ? " heads=sampled" : " heads=argmax";
     if (ctx->prefill_rows >= 2)
         d += " prefill=chunks of " + std::to_string(ctx->prefill_rows) + " rows (" +
-             (ctx->prefill_tile_attn && attn_mma_ok(ctx) ? "attn_prefill_kernel" : "per-row attention") + ")";
+             (ctx->prefill_attn != 1 && attn_mma_ok(ctx) ? "attn_prefill_kernel" : "per-row attention") + ")";
     snprintf(h_buf, cap, "%s", d.c_str());
     return PIPO_OK;
 }
