@@ -175,6 +175,8 @@ struct pipo_ctx {
     int rows = 0;                     // activation rows of the enqueue in progress (0: B, one per sequence)
     int max_rows = 0;                 // rows the activation buffers hold: max(max_batch, prefill_rows)
     int prefill_rows = 0;             // rows of a prefill chunk (positions x sequences; 0: one position at a time)
+    bool prefill_auto = false;        // prefill_rows not set by the caller: chunks by the batch (prefill_chunk_rows)
+    bool rows_fp32 = false;           // the chunk in progress keeps the fp32 products of a single sequence's GEMVs
     int prefill_attn = 0;             // chunk attention: 0 by size, 1 row by row, 2 causal tiles (attn_prefill_kernel)
     // sampling in both heads (pipo_set_sampler; greedy when off)
     bool samp_on = false;
@@ -297,6 +299,7 @@ constexpr size_t kXsBudget = 100 * 1024;      // fp32 bytes of the longest GEMV 
 // cached keys and values); longer slices take the register ring alone
 constexpr size_t kAttnStageMax = 160 * 1024;
 constexpr int kMaxPrefillRows = 2048;         // rows of a prefill chunk (PIPO_PREFILL_ROWS)
+constexpr int kAutoRows = 512;                // ... that the library chooses by itself
 constexpr size_t kBlkSmemMax = (size_t)kBlkKMax * kBlkNB * 4 + (size_t)kBlkSeg * 32 * 4;
 constexpr size_t kStreamBudget = 200 * 1024;  // staged-input bytes per streaming GEMV block
 
@@ -750,6 +753,7 @@ pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int spl
 
 bool tc_eligible(const pipo_ctx* ctx, const GemvParams& p) {
     const int rows = p.N * (p.epi == EPI_SWIGLU ? 2 : 1);
+    if (ctx->rows_fp32) return false;
     // decode batches above 128 keep the fp32 products of the CUDA-core GEMV;
     // prefill chunks may be as tall as their buffers
     const int most = ctx->rows > ctx->B ? ctx->tc_bn_max : std::min(ctx->tc_bn_max, 128);
@@ -1488,9 +1492,10 @@ pipo_status enqueue_prefill_chunk(pipo_ctx* ctx, bool regular, int j0, int C) {
         return fail(ctx, PIPO_EINVAL, "prefill chunk of %d rows (at most %d)", R, ctx->max_rows);
     struct RowsGuard {
         pipo_ctx* c;
-        ~RowsGuard() { c->rows = 0; }
+        ~RowsGuard() { c->rows = 0; c->rows_fp32 = false; }
     } guard{ctx};
     ctx->rows = R;
+    ctx->rows_fp32 = ctx->prefill_auto && B < ctx->tc_min_b;
     ctx->tc_shallow = attn_is_long(ctx);
     const bool bf = c.dtype == 1;
     if (regular) {
@@ -1550,9 +1555,15 @@ pipo_status enqueue_prefill_chunk(pipo_ctx* ctx, bool regular, int j0, int C) {
 // two rounds, and 1792 rows 70 tiles, one.  Chosen: the n * 256 rows of the
 // least rounds x K per row, a chunk's launches standing for kChunkK inputs
 // (about 40 us per block at 0.6 us per 64 inputs of a round).
+//
+// When the caller has not set the rows: a batch whose steps run on the tensor
+// cores takes chunks of up to kAutoRows on them, and one whose steps keep
+// fp32 products (a single sequence, fp32 models) one weight pass of the
+// row-block GEMV, eight rows.
 constexpr int kChunkK = 4300;
 int prefill_chunk_rows(const pipo_ctx* ctx) {
     const pipo_config& c = ctx->cfg;
+    if (ctx->prefill_auto && (c.dtype != 1 || ctx->B < ctx->tc_min_b)) return kBlkNB;
     if (ctx->prefill_rows < 2 * kPairN || c.dtype != 1) return ctx->prefill_rows;
     const int pairs = std::max(1, pair_max_clusters()), qd = c.n_q_heads * c.head_dim, kd = c.n_kv_heads * c.head_dim;
     const int shp[4][2] = {{qd + 2 * kd, c.hidden}, {c.hidden, qd}, {2 * c.ffn, c.hidden}, {c.hidden, c.ffn}};
@@ -1823,8 +1834,12 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         // activations and state
         const int qd = c.n_q_heads * DH, kd = c.n_kv_heads * DH;
         // prefill chunks: PIPO_PREFILL_ROWS=<rows> (positions x sequences per
-        // chunk, at most kMaxPrefillRows; 0 or unset: one position at a time)
+        // chunk, at most kMaxPrefillRows; 0: one position at a time; unset: by
+        // the batch, see prefill_chunk_rows)
+        if (const char* ev = getenv("PIPO_TC_MIN_BATCH")) ctx->tc_min_b = std::max(1, atoi(ev));
         if (const char* ev = getenv("PIPO_PREFILL_ROWS")) ctx->prefill_rows = std::min(kMaxPrefillRows, std::max(0, atoi(ev)));
+        else ctx->prefill_auto = true;
+        if (ctx->prefill_auto) ctx->prefill_rows = c.dtype == 1 && MB >= ctx->tc_min_b ? kAutoRows : kBlkNB;
         if (const char* ev = getenv("PIPO_PREFILL_ATTN")) ctx->prefill_attn = strcmp(ev, "tile") == 0 ? 2 : 1;
         const int MR = std::max(MB, ctx->prefill_rows);
         ctx->max_rows = MR;
@@ -1849,10 +1864,9 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         CK(cudaMemset(ctx->counters, 0, (size_t)MB * c.n_kv_heads * 4));
         TRY(dalloc(ctx, &ctx->am, (size_t)2 * MB * 8));
         // tensor-core projections: the bf16 activation tile
-        if (const char* ev = getenv("PIPO_TC_MIN_BATCH")) ctx->tc_min_b = std::max(1, atoi(ev));
         if (const char* ev = getenv("PIPO_ATTN_MMA_MIN_BATCH")) ctx->attn_mma_min_b = std::max(1, atoi(ev));
         if (const char* ev = getenv("PIPO_TC_SPLITS")) ctx->tc_splits = std::max(0, atoi(ev));
-        if (c.dtype == 1 && MR >= ctx->tc_min_b) {
+        if (c.dtype == 1 && (ctx->prefill_auto ? MB : MR) >= ctx->tc_min_b) {
             ctx->tc_bn_max = tc_bn(std::max(std::min(MB, 128), ctx->prefill_rows));
             ctx->tc_kmax = std::max({2 * (int)H, qd, c.ffn});
             TRY(dalloc(ctx, &ctx->tc_xb, (size_t)2 * ctx->tc_bn_max * ctx->tc_kmax * 2));
@@ -2771,7 +2785,7 @@ pipo_status pipo_describe_step(const pipo_ctx* ctx, char* h_buf, size_t cap) {
     // decoding mode, heads and prefill arrangement
     d += ctx->regular ? " mode=regular" : " mode=pair";
     d += ctx->samp_on ? " heads=sampled" : " heads=argmax";
-    if (ctx->prefill_rows >= 2)
+    if (ctx->prefill_rows >= 2 && !ctx->prefill_auto)
         d += " prefill=chunks of " + std::to_string(ctx->prefill_rows) + " rows (" +
              (ctx->prefill_attn != 1 && attn_mma_ok(ctx) ? "attn_prefill_kernel" : "per-row attention") + ")";
     snprintf(h_buf, cap, "%s", d.c_str());
