@@ -109,6 +109,7 @@ void* k_pick_append_rows(bool bf, int DH) {
     return nullptr;
 }
 
+cudaError_t k_error_word_attn(const unsigned** p) { return unit_error_word(p); }
 cudaError_t k_take_error_attn(unsigned* code, unsigned* info) { return take_unit_error(code, info); }
 
 #ifdef PIPO_TRACE

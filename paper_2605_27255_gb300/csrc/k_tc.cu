@@ -46,6 +46,7 @@ void* k_pick_pair() { return reinterpret_cast<void*>(&gemm_pair_kernel<kPairN>);
 
 void* k_pick_prep_bf16() { return reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16>); }
 
+cudaError_t k_error_word_tc(const unsigned** p) { return unit_error_word(p); }
 cudaError_t k_take_error_tc(unsigned* code, unsigned* info) { return take_unit_error(code, info); }
 
 // Self-test of the bounded wait (site 90): thread 0 waits, with a limit of

@@ -20,6 +20,7 @@ void* k_pick_stream_f32(int nb, int ru, bool rows);
 void* k_pick_tcv(int bh, bool deep, bool fused);    // gemm_tcf_kernel (fused) / gemm_tc_kernel
 void* k_pick_pair();                                // gemm_pair_kernel
 void* k_pick_prep_bf16();                           // prep_bf16_kernel<bf16>
+cudaError_t k_error_word_tc(const unsigned** p);      // device address of the unit's error word
 cudaError_t k_take_error_tc(unsigned* code, unsigned* info);
 void* k_pick_wait_selftest();                       // wait_selftest_kernel (reports through k_take_error_tc)
 
@@ -32,6 +33,7 @@ void* k_pick_attn_mma_flat(int G);                  // attn_mma_kernel, uncluste
 void* k_pick_attn_prefill(int G);                   // attn_prefill_kernel
 void* k_pick_rope_append(bool bf, int DH);          // rope_append_kernel
 void* k_pick_append_rows(bool bf, int DH);          // append_rows_kernel
+cudaError_t k_error_word_attn(const unsigned** p);      // device address of the unit's error word
 cudaError_t k_take_error_attn(unsigned* code, unsigned* info);
 
 #ifdef PIPO_TRACE

@@ -438,7 +438,25 @@ struct StepState {
     uint32_t* presence;
     int presence_w;
     int32_t* samp_step;
+    // mapped host memory: the outputs once more, and the device error words of
+    // the units whose kernels wait, so that a synchronous step needs no copy
+    // and no further call to read them
+    int32_t* host_tokens;  // [B,2]
+    int32_t* host_nacc;    // [B]
+    unsigned* host_err;
+    const unsigned* err_word[2];
 };
+
+// Outputs of sequence b at the end of a step (one thread).
+__device__ __forceinline__ void publish_step(const StepState& st, int b, int xb, int xd, int accept) {
+    st.out_tokens[2 * b] = st.host_tokens[2 * b] = xb;
+    st.out_tokens[2 * b + 1] = st.host_tokens[2 * b + 1] = xd;
+    st.out_nacc[b] = st.host_nacc[b] = accept;
+    if (b == 0) {
+        const unsigned e = __ldcg(st.err_word[0]) | __ldcg(st.err_word[1]);
+        if (e) *st.host_err = e;
+    }
+}
 
 // Confidence c = sigmoid(W2 . t) with t = SiLU(W1 RMSNorm([h_b; h_d])) computed
 // by the preceding GEMV; acceptance; next pending pair; counters.  grid B,
@@ -489,9 +507,7 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(const float* __r
     const float c = 1.0f / (1.0f + expf(-s));
     const int accept = (force == 1) ? 1 : (force == 2) ? 0 : (c >= tau ? 1 : 0);
     const int xb = argmax_row(st.am_b[b]), xd = argmax_row(st.am_d[b]);
-    st.out_tokens[2 * b] = xb;
-    st.out_tokens[2 * b + 1] = accept ? xd : -1;
-    st.out_nacc[b] = accept;
+    publish_step(st, b, xb, accept ? xd : -1, accept);
     st.pending[2 * b] = xb;
     st.pending[2 * b + 1] = accept ? xd : -1;
     st.n_pos[b] += 1;

@@ -57,6 +57,16 @@ __global__ void advance_kernel(int32_t* n_pos, int B, int by) {
 }
 
 
+// n integers from the launch's own parameters: a small host array reaches the
+// device in stream order without a staging buffer or a synchronisation.
+constexpr int kIntPack = 256;
+struct IntPack {
+    int32_t v[kIntPack];
+};
+__global__ void set_ints_kernel(int32_t* dst, const __grid_constant__ IntPack src, int n) {
+    if ((int)threadIdx.x < n) dst[threadIdx.x] = src.v[threadIdx.x];
+}
+
 // Regular decoding, end of a step: the LM-head argmax is the output token and
 // the next input (slot 1 stays PAD, nothing is drafted), one more cache entry,
 // one more emitted token.  grid B, any block size.
@@ -68,9 +78,7 @@ __global__ void regular_accept_kernel(StepState st, int H, const float* h) {
         for (int k = threadIdx.x; k < H; k += blockDim.x) st.dbg_hb[(size_t)b * H + k] = h[(size_t)b * H + k];
     if (threadIdx.x != 0) return;
     const int xb = argmax_row(st.am_b[b]);
-    st.out_tokens[2 * b] = xb;
-    st.out_tokens[2 * b + 1] = -1;
-    st.out_nacc[b] = 0;
+    publish_step(st, b, xb, -1, 0);
     st.pending[2 * b] = xb;
     st.pending[2 * b + 1] = -1;
     st.n_pos[b] += 1;
@@ -128,6 +136,12 @@ struct pipo_ctx {
     int tc_splits = 0;              // forced K splits (0: automatic)
 
     int32_t *pending = nullptr, *n_pos = nullptr, *out_tokens = nullptr, *out_nacc = nullptr;
+    // mapped host memory, written by the kernel that ends a step: tokens
+    // [max_batch][2], acceptances [max_batch], device error words (or'ed)
+    int32_t* host_blk = nullptr;
+    int32_t *host_tokens = nullptr, *host_nacc = nullptr;
+    unsigned* host_err = nullptr;
+    const unsigned* err_word[2] = {nullptr, nullptr};
     long long* emitted = nullptr;
     float *dbg_lb = nullptr, *dbg_ld = nullptr, *dbg_conf = nullptr, *dbg_hb = nullptr, *dbg_hd = nullptr;
     int32_t *dbg_xb = nullptr, *dbg_xd = nullptr;
@@ -1415,6 +1429,8 @@ pipo_status enqueue_position(pipo_ctx* ctx, Mode mode, int j) {
     StepState st{};
     st.pending = ctx->pending; st.n_pos = ctx->n_pos; st.emitted = ctx->emitted;
     st.out_tokens = ctx->out_tokens; st.out_nacc = ctx->out_nacc;
+    st.host_tokens = ctx->host_tokens; st.host_nacc = ctx->host_nacc; st.host_err = ctx->host_err;
+    st.err_word[0] = ctx->err_word[0]; st.err_word[1] = ctx->err_word[1];
     st.am_b = am_b; st.am_d = am_d;
     if (c.debug) {
         st.dbg_conf = ctx->dbg_conf; st.dbg_hb = ctx->dbg_hb; st.dbg_hd = ctx->dbg_hd;
@@ -1468,6 +1484,8 @@ pipo_status enqueue_regular(pipo_ctx* ctx, Mode mode, int j) {
     StepState st{};
     st.pending = ctx->pending; st.n_pos = ctx->n_pos; st.emitted = ctx->emitted;
     st.out_tokens = ctx->out_tokens; st.out_nacc = ctx->out_nacc;
+    st.host_tokens = ctx->host_tokens; st.host_nacc = ctx->host_nacc; st.host_err = ctx->host_err;
+    st.err_word[0] = ctx->err_word[0]; st.err_word[1] = ctx->err_word[1];
     st.am_b = ctx->am; st.am_d = ctx->am;
     if (c.debug) { st.dbg_hb = ctx->dbg_hb; st.dbg_xb = ctx->dbg_xb; }
     int Hv = H;
@@ -1701,6 +1719,34 @@ pipo_status check_device_error(pipo_ctx* ctx) {
                 e, info[0], info[1], info[2], info[3]);
 }
 
+// After a synchronised step or prefill: the error words as the step's last
+// kernel saw them; only when one is set are the units asked for the wait.
+pipo_status check_step_error(pipo_ctx* ctx) {
+    const unsigned e = *static_cast<volatile unsigned*>(ctx->host_err);
+    if (!e) return PIPO_OK;
+    *ctx->host_err = 0u;
+    TRY(check_device_error(ctx));
+    return fail(ctx, PIPO_ECUDA, "device wait timed out (code %u): results of this step are invalid", e);
+}
+
+// The outputs of the last step or prefill, once the stream is synchronised.
+void read_outputs(const pipo_ctx* ctx, int B, int32_t* h_tokens, int32_t* h_n_accepted) {
+    if (h_tokens) memcpy(h_tokens, ctx->host_tokens, (size_t)B * 8);
+    if (h_n_accepted) memcpy(h_n_accepted, ctx->host_nacc, (size_t)B * 4);
+}
+
+// n host integers into device memory, in stream order; h is read before it returns.
+pipo_status put_ints(pipo_ctx* ctx, int32_t* dst, const int32_t* h, int n) {
+    for (int i = 0; i < n; i += kIntPack) {
+        IntPack pk;
+        const int m = std::min(kIntPack, n - i);
+        memcpy(pk.v, h + i, (size_t)m * 4);
+        set_ints_kernel<<<1, kIntPack, 0, ctx->stream>>>(dst + i, pk, m);
+        CK(cudaGetLastError());
+    }
+    return PIPO_OK;
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ C ABI
@@ -1717,6 +1763,7 @@ void pipo_free(pipo_ctx* ctx) {
     drop_graph(ctx);
     for (cudaEvent_t e : ctx->prof_ev) cudaEventDestroy(e);
     for (void* p : ctx->allocs) cudaFree(p);
+    if (ctx->host_blk) cudaFreeHost(ctx->host_blk);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
     delete ctx;
 }
@@ -1875,6 +1922,18 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         TRY(dalloc(ctx, &ctx->n_pos, (size_t)MB * 4));
         TRY(dalloc(ctx, &ctx->out_tokens, (size_t)MB * 2 * 4));
         TRY(dalloc(ctx, &ctx->out_nacc, (size_t)MB * 4));
+        const size_t hb_bytes = ((size_t)MB * 3 + 1) * 4;
+        if (cudaHostAlloc(reinterpret_cast<void**>(&ctx->host_blk), hb_bytes, cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->host_blk = nullptr;
+            return fail(ctx, PIPO_ENOMEM, "cudaHostAlloc(%zu bytes)", hb_bytes);
+        }
+        memset(ctx->host_blk, 0, hb_bytes);
+        ctx->host_tokens = ctx->host_blk;
+        ctx->host_nacc = ctx->host_blk + 2 * MB;
+        ctx->host_err = reinterpret_cast<unsigned*>(ctx->host_blk + 3 * MB);
+        CK(k_error_word_attn(&ctx->err_word[0]));
+        CK(k_error_word_tc(&ctx->err_word[1]));
         TRY(dalloc(ctx, &ctx->emitted, (size_t)MB * 8));
         CK(cudaMemset(ctx->n_pos, 0, (size_t)MB * 4));
         CK(cudaMemset(ctx->emitted, 0, (size_t)MB * 8));
@@ -2101,12 +2160,11 @@ pipo_status pipo_prefill(pipo_ctx* ctx, int32_t batch, const int32_t* h_ids, int
         }
     }
     ctx->launches = saved;
-    if (h_tokens) CK(cudaMemcpyAsync(h_tokens, ctx->out_tokens, (size_t)batch * 8, cudaMemcpyDeviceToHost, ctx->stream));
-    if (h_n_accepted) CK(cudaMemcpyAsync(h_n_accepted, ctx->out_nacc, (size_t)batch * 4, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    read_outputs(ctx, batch, h_tokens, h_n_accepted);
     ctx->h_len.assign(batch, N);
     ctx->prefilled = true;
-    return check_device_error(ctx);
+    return check_step_error(ctx);
 }
 
 }  // extern "C"
@@ -2118,7 +2176,7 @@ namespace {
 // are scratch shared by all slots).  Restored on destruction.
 struct SlotView {
     pipo_ctx* c;
-    int32_t *n_pos, *pending, *out_tokens, *out_nacc, *block_table, *dbg_xb, *dbg_xd;
+    int32_t *n_pos, *pending, *out_tokens, *out_nacc, *block_table, *dbg_xb, *dbg_xd, *host_tokens, *host_nacc;
     long long* emitted;
     float *dbg_lb, *dbg_ld, *dbg_conf, *dbg_hb, *dbg_hd, *samp_u;
     uint32_t* presence;
@@ -2128,6 +2186,8 @@ struct SlotView {
         block_table = ctx->block_table; dbg_xb = ctx->dbg_xb; dbg_xd = ctx->dbg_xd; emitted = ctx->emitted;
         dbg_lb = ctx->dbg_lb; dbg_ld = ctx->dbg_ld; dbg_conf = ctx->dbg_conf; dbg_hb = ctx->dbg_hb;
         dbg_hd = ctx->dbg_hd; samp_u = ctx->samp_u; presence = ctx->presence;
+        host_tokens = ctx->host_tokens; host_nacc = ctx->host_nacc;
+        ctx->host_tokens += 2 * s; ctx->host_nacc += s;
         ctx->n_pos += s; ctx->pending += 2 * s; ctx->out_tokens += 2 * s; ctx->out_nacc += s; ctx->emitted += s;
         ctx->block_table += (size_t)s * ctx->blocks_per_seq;
         if (ctx->dbg_lb) {
@@ -2142,6 +2202,7 @@ struct SlotView {
         c->block_table = block_table; c->dbg_xb = dbg_xb; c->dbg_xd = dbg_xd; c->emitted = emitted;
         c->dbg_lb = dbg_lb; c->dbg_ld = dbg_ld; c->dbg_conf = dbg_conf; c->dbg_hb = dbg_hb; c->dbg_hd = dbg_hd;
         c->samp_u = samp_u; c->presence = presence;
+        c->host_tokens = host_tokens; c->host_nacc = host_nacc;
     }
 };
 
@@ -2214,12 +2275,11 @@ pipo_status pipo_regular_prefill(pipo_ctx* ctx, int32_t batch, const int32_t* h_
     ctx->launches = saved;
     // the prefill's token is the first output, not a decode step's
     CK(cudaMemsetAsync(ctx->emitted, 0, (size_t)batch * 8, ctx->stream));
-    if (h_tokens) CK(cudaMemcpyAsync(h_tokens, ctx->out_tokens, (size_t)batch * 8, cudaMemcpyDeviceToHost, ctx->stream));
-    if (h_n_accepted) CK(cudaMemcpyAsync(h_n_accepted, ctx->out_nacc, (size_t)batch * 4, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    read_outputs(ctx, batch, h_tokens, h_n_accepted);
     ctx->h_len.assign(batch, N);
     ctx->prefilled = true;
-    return check_device_error(ctx);
+    return check_step_error(ctx);
 }
 
 }  // extern "C"
@@ -2247,10 +2307,9 @@ pipo_status step_async(pipo_ctx* ctx, bool regular, int32_t* d_tokens, int32_t* 
 
 pipo_status step_sync(pipo_ctx* ctx, bool regular, int32_t* h_tokens, int32_t* h_n_accepted) {
     TRY(step_async(ctx, regular, nullptr, nullptr));
-    if (h_tokens) CK(cudaMemcpyAsync(h_tokens, ctx->out_tokens, (size_t)ctx->B * 8, cudaMemcpyDeviceToHost, ctx->stream));
-    if (h_n_accepted) CK(cudaMemcpyAsync(h_n_accepted, ctx->out_nacc, (size_t)ctx->B * 4, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    return check_device_error(ctx);
+    read_outputs(ctx, ctx->B, h_tokens, h_n_accepted);
+    return check_step_error(ctx);
 }
 
 }  // namespace
@@ -2297,7 +2356,7 @@ pipo_status pipo_decode_steps(pipo_ctx* ctx, int32_t n_steps, int32_t* h_tokens,
         if (h_tokens) std::copy(o, o + 2 * B, h_tokens + (size_t)i * B * 2);
         if (h_n_accepted) std::copy(o + 2 * B, o + 3 * B, h_n_accepted + (size_t)i * B);
     }
-    return check_device_error(ctx);
+    return check_step_error(ctx);
 }
 
 pipo_status pipo_regular_step_async(pipo_ctx* ctx, int32_t* d_tokens) {
@@ -2315,8 +2374,7 @@ pipo_status pipo_rollback(pipo_ctx* ctx, const int32_t* h_n_pairs) {
         if (h_n_pairs[b] < 0 || h_n_pairs[b] > ctx->h_len[b])
             return fail(ctx, PIPO_EINVAL, "sequence %d: rollback to %d of %d entries", b, h_n_pairs[b], ctx->h_len[b]);
     CK(cudaSetDevice(ctx->dev));
-    CK(cudaMemcpyAsync(ctx->n_pos, h_n_pairs, (size_t)ctx->B * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    TRY(put_ints(ctx, ctx->n_pos, h_n_pairs, ctx->B));
     for (int b = 0; b < ctx->B; ++b) ctx->h_len[b] = h_n_pairs[b];
     return PIPO_OK;
 }
@@ -2330,8 +2388,7 @@ pipo_status pipo_set_pending(pipo_ctx* ctx, const int32_t* h_pairs) {
             return fail(ctx, PIPO_EINVAL, "sequence %d: pending pair out of range", b);
     }
     CK(cudaSetDevice(ctx->dev));
-    CK(cudaMemcpyAsync(ctx->pending, h_pairs, (size_t)ctx->B * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    TRY(put_ints(ctx, ctx->pending, h_pairs, 2 * ctx->B));
     return PIPO_OK;
 }
 

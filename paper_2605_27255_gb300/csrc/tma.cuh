@@ -27,6 +27,14 @@ static __device__ unsigned int g_pipo_error_info[4];
 constexpr unsigned kErrWaitTimeout = 1u;
 constexpr unsigned long long kWaitNs = 2000000000ull;  // give up after 2 s of waiting
 
+// Host: device address of this translation unit's error word.
+static inline cudaError_t unit_error_word(const unsigned** p) {
+    void* a = nullptr;
+    const cudaError_t e = cudaGetSymbolAddress(&a, g_pipo_error);
+    *p = static_cast<const unsigned*>(a);
+    return e;
+}
+
 // Host: read and clear this translation unit's error word and wait record.
 static inline cudaError_t take_unit_error(unsigned* code, unsigned info[4]) {
     cudaError_t e = cudaMemcpyFromSymbol(code, g_pipo_error, sizeof(unsigned));
