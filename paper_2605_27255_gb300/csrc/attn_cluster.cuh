@@ -87,6 +87,11 @@ struct AttnParams {
     float* part_o;
     float* part_ml;
     unsigned* counters;
+    // balanced unclustered form (attn_mma_kernel, slots > 0): grid x counts
+    // slots that every CTA maps to a sequence and a split by the cached
+    // lengths (attn_slot_map); the partial of query head h in slot i is at
+    // [h * slots + i]
+    int slots;
     // staged form (stage_max > 0): the CTA's whole slice of cached keys and
     // values is copied to shared memory (bulk copies, one per page run and
     // tensor) before the dependency wait; stage_max entries fit

@@ -164,13 +164,68 @@ __device__ __forceinline__ void mma_rows8(float (&d)[4], uint32_t a0, uint32_t a
         : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
 }
 
+// The balanced split of sequences of different lengths: with the smallest
+// chunk c such that every sequence b cut into ceil((n_pos[b] + 1) / c) splits
+// needs at most `slots` of them, slot i is split s of n of sequence b, whose
+// first slot is `base` (b = -1: none).  Every lane of a warp gets the same answer.
+constexpr int kSlotSeqs = 128;  // sequences: four per lane
+struct SlotMap {
+    int b, s, n, base;
+};
+__device__ __forceinline__ SlotMap attn_slot_map(const int32_t* n_pos, int nseq, int slots, int slot) {
+    const int lane = threadIdx.x & 31;
+    int len[kSlotSeqs / 32], total = 0, most = 0;
+#pragma unroll
+    for (int k = 0; k < kSlotSeqs / 32; ++k) {
+        const int i = k * 32 + lane;
+        len[k] = i < nseq ? n_pos[i] + 1 : 0;
+        total += len[k];
+        most = max(most, len[k]);
+    }
+    total = __reduce_add_sync(0xffffffffu, total);
+    int hi = __reduce_max_sync(0xffffffffu, most), lo = max(1, total / slots);
+    while (lo < hi) {
+        const int c = (lo + hi) >> 1;
+        int n = 0;
+#pragma unroll
+        for (int k = 0; k < kSlotSeqs / 32; ++k) n += (len[k] + c - 1) / c;
+        if ((int)__reduce_add_sync(0xffffffffu, n) <= slots) hi = c; else lo = c + 1;
+    }
+    SlotMap m{-1, 0, 0, 0};
+    int pre = 0;
+#pragma unroll
+    for (int k = 0; k < kSlotSeqs / 32; ++k) {
+        const int n = (len[k] + lo - 1) / lo;
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const int base = pre + incl - n;
+        const unsigned hit = __ballot_sync(0xffffffffu, slot >= base && slot < base + n);
+        if (hit) {
+            const int src = __ffs(hit) - 1;
+            m.b = k * 32 + src;
+            m.n = __shfl_sync(0xffffffffu, n, src);
+            m.base = __shfl_sync(0xffffffffu, base, src);
+            m.s = slot - m.base;
+        }
+        pre += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    return m;
+}
+
 // tmK, tmV: this layer's K and V cache as [blocks * n_kv * page][d_h] bf16,
 // boxes of 64 dims x 16 rows, 128-byte swizzle
 // FLAT: no cluster; the grid's x dimension splits the entries (S = gridDim.x
 // CTAs per (row, kv head)), each CTA writes its partial to the global
 // scratch (AttnParams::part_o, part_ml) and the last of a (row, kv head) to
 // arrive (AttnParams::counters) merges the S partials in split order: any
-// split count, so that long caches fill the GPU evenly.
+// split count, so that long caches fill the GPU evenly.  With
+// AttnParams::slots the splits follow the lengths: a batch of sequences of
+// different ages otherwise waits for the longest one's CTAs (4B, B = 16,
+// 161 .. 2415 entries: 37.6 us per launch in clusters of two, 29.8 so).
 template <int G, bool FLAT = false, int ST = kMmaStages>
 __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, const __grid_constant__ CUtensorMap tmK,
                                                                const __grid_constant__ CUtensorMap tmV) {
@@ -199,10 +254,19 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
 
     pdl_launch();
     cg::cluster_group cluster = cg::this_cluster();
-    const int s = FLAT ? (int)blockIdx.x : (int)cluster.block_rank();
-    const int CS = FLAT ? (int)gridDim.x : (int)cluster.num_blocks();
+    int s = FLAT ? (int)blockIdx.x : (int)cluster.block_rank();
+    int CS = FLAT ? (int)gridDim.x : (int)cluster.num_blocks();
+    int row = blockIdx.z, slot0 = 0;
+    if (FLAT && p.slots > 0) {  // the lengths change only between steps: read before the dependency wait
+        const SlotMap sm = attn_slot_map(p.n_pos, p.nseq, p.slots, (int)blockIdx.x);
+        if (sm.b < 0) return;
+        row = sm.b;
+        s = sm.s;
+        CS = sm.n;
+        slot0 = sm.base;
+    }
     __shared__ int last_cta;
-    const int g = blockIdx.y, row = blockIdx.z;
+    const int g = blockIdx.y;
     const int b = row % p.nseq;        // sequence: its block table and length
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_kv = p.kv.n_kv, n_q = n_kv * G;
@@ -443,6 +507,10 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
         cluster_wait_acquire();  // rank 0's receive barrier is initialised
         slot = cluster.map_shared_rank(rcv, 0) + (size_t)s * kMmaRcvSlot;
     }
+    // unclustered: the partials of this (row, kv head), head hh, split 0
+    auto part_at = [&](int hh) {
+        return p.slots > 0 ? (size_t)(g * G + hh) * p.slots + slot0 : (size_t)(row * n_q + g * G + hh) * CS;
+    };
     // four consecutive output dims per thread (16-byte stores, also into rank 0)
     for (int i4 = threadIdx.x; i4 < G * DH / 4; i4 += blockDim.x) {
         const int hh = (4 * i4) / DH, t = (4 * i4) % DH;
@@ -458,8 +526,8 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
             const float4 v = *reinterpret_cast<const float4*>(w < NW ? wpart(w) + hh * DH + t : &wo_new[hh][t]);
             Ov.x += v.x * f; Ov.y += v.y * f; Ov.z += v.z * f; Ov.w += v.w * f;
         }
-        if (FLAT) {
-            const size_t pi = (size_t)(row * n_q + g * G + hh) * CS + s;
+        if (FLAT && CS > 1) {
+            const size_t pi = part_at(hh) + s;
             __stcg(reinterpret_cast<float4*>(p.part_o + pi * DH + t), Ov);
             if (t == 0) {
                 p.part_ml[pi * 2] = M;
@@ -479,6 +547,7 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
     }
     PIPO_TR(if (threadIdx.x == 0) tr_s[2] = trace_now();)
     if constexpr (FLAT) {
+        if (CS == 1) return;
         // the last CTA of (row, kv head) to arrive merges the CS partials in split order
         __threadfence();
         __syncthreads();
@@ -495,7 +564,7 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
         float* fs = ms + G * CS;
         for (int i = threadIdx.x; i < G * CS; i += blockDim.x) {
             const int hh = i / CS, r2 = i % CS;
-            const size_t pi = (size_t)(row * n_q + g * G + hh) * CS + r2;
+            const size_t pi = part_at(hh) + r2;
             ms[i] = __ldcg(p.part_ml + pi * 2);
             fs[i] = __ldcg(p.part_ml + pi * 2 + 1);
         }
@@ -515,7 +584,7 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
         __syncthreads();
         for (int i4 = threadIdx.x; i4 < G * DH / 4; i4 += blockDim.x) {
             const int hh = (4 * i4) / DH, t = (4 * i4) % DH;
-            const float* po = p.part_o + (size_t)(row * n_q + g * G + hh) * CS * DH + t;
+            const float* po = p.part_o + part_at(hh) * DH + t;
             float4 Ov = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int r0 = 0; r0 < CS; r0 += 4) {
                 float4 ov[4];

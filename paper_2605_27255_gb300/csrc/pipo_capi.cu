@@ -208,6 +208,7 @@ struct pipo_ctx {
     std::vector<int32_t> h_len;
     cudaGraphExec_t graph = nullptr;
     int graph_B = -1;
+    std::vector<int32_t> plan_lens;   // the cached lengths at its capture
     double plan_len = -1.0;           // mean cached length the step graph's launch plan was made for
     bool graph_regular = false;       // the captured step is a regular-decoding step
     int launches = 0;
@@ -1091,6 +1092,41 @@ int attn_mma_flat_splits(const pipo_ctx* ctx, int R) {
     return std::max(1, std::min(S, kFlatMaxSplits));
 }
 
+// Slots per kv head of the balanced unclustered attention (splits by the
+// cached lengths, attn_slot_map), or 0: for a batch of different lengths whose
+// longest slice would otherwise set the launch's time.  One wave of two CTAs
+// per SM; taken when the balanced slices, with kSlotCost entries for the
+// merge through global memory, are shorter than the longest sequence's slice
+// in the cluster of `cs` CTAs (8 4B-wide layers,
+// B = 16, 161 .. 2415 entries: 0.98 -> 0.91 ms per step).
+constexpr int kSlotCost = 128;
+int attn_mma_slots(const pipo_ctx* ctx, int R, int cs) {
+    const std::vector<int32_t>& lens = ctx->graph ? ctx->plan_lens : ctx->h_len;
+    if (R != ctx->B || R < 2 || R > kSlotSeqs || (int)lens.size() < R) return 0;
+    const int slots = 2 * ctx->sms / ctx->cfg.n_kv_heads;
+    if (slots < R) return 0;
+    long long total = 0;
+    int most = 0;
+    for (int b = 0; b < R; ++b) {
+        total += lens[b] + 1;
+        most = std::max(most, lens[b] + 1);
+    }
+    int lo = (int)std::max<long long>(1, total / slots), hi = most;
+    while (lo < hi) {
+        const int c = (lo + hi) / 2;
+        int n = 0;
+        for (int b = 0; b < R; ++b) n += (lens[b] + c) / c;
+        if (n <= slots) hi = c; else lo = c + 1;
+    }
+    return lo + kSlotCost < (most + cs - 1) / cs ? slots : 0;
+}
+// ... against the uniform splits the batch would take otherwise
+int attn_balanced_slots(const pipo_ctx* ctx, int R) {
+    if (ctx->attn_cs_force) return 0;
+    const int flat = attn_mma_flat_splits(ctx, R);
+    return attn_mma_slots(ctx, R, flat > 0 ? flat : attn_cluster_size(ctx, R));
+}
+
 // Long attention: the cached K/V bytes of a layer are at least six times the
 // QKV weight bytes (cached lengths at graph capture).  Then every projection
 // takes the two-per-SM ring, whose shared memory leaves room for a
@@ -1218,6 +1254,14 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
             void* pargs[] = {&ap, &C, &ctx->kv_tm[2 * cache_layer], &ctx->kv_tm[2 * cache_layer + 1]};
             TRY(launch_ex(ctx, fn, dim3((C + TP - 1) / TP, c.n_kv_heads, ctx->B), dim3(kPfThreads),
                           prefill_attn_smem(), pargs));
+        } else if (attn_use_mma(ctx, R) && !chunk && attn_balanced_slots(ctx, R) > 0) {
+            ap.part_o = ctx->part_o;
+            ap.part_ml = ctx->part_ml;
+            ap.counters = ctx->counters;
+            ap.slots = attn_balanced_slots(ctx, R);
+            void* margs[] = {&ap, &ctx->kv_tm[2 * cache_layer], &ctx->kv_tm[2 * cache_layer + 1]};
+            TRY(launch_ex(ctx, k_pick_attn_mma_flat(G), dim3(ap.slots, c.n_kv_heads), dim3(kMmaThreads),
+                          mma_attn_smem(1), margs));
         } else if (attn_use_mma(ctx, R) && !chunk && attn_mma_flat_splits(ctx, R) > 0) {
             // long caches: unclustered splits, one wave of two CTAs per SM
             ap.part_o = ctx->part_o;
@@ -1655,6 +1699,7 @@ pipo_status ensure_graph(pipo_ctx* ctx) {
     ctx->graph_B = ctx->B;
     ctx->graph_regular = ctx->regular;
     ctx->plan_len = plan_len;
+    ctx->plan_lens = ctx->h_len;
     return PIPO_OK;
 }
 
@@ -1905,6 +1950,8 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
         for (int b = 1; b <= MB; ++b) parts = std::max(parts, (size_t)b * c.n_q_heads * attn_splits(ctx, b));
         // the unclustered tensor-core attention: rows x n_kv < 2 sms / 8, at most kFlatMaxSplits splits
         parts = std::max(parts, (size_t)(2 * ctx->sms / 8 + 1) * (c.n_q_heads / c.n_kv_heads) * kFlatMaxSplits);
+        // ... the balanced one: a partial per query head and slot
+        parts = std::max(parts, (size_t)c.n_q_heads * (2 * ctx->sms / c.n_kv_heads + 1));
         TRY(dalloc(ctx, &ctx->part_o, parts * DH * 4));
         TRY(dalloc(ctx, &ctx->part_ml, parts * 2 * 4));
         TRY(dalloc(ctx, &ctx->counters, (size_t)MB * c.n_kv_heads * 4));
@@ -2827,12 +2874,14 @@ pipo_status pipo_describe_step(const pipo_ctx* ctx, char* h_buf, size_t cap) {
                               cuda_core + ")";
     else proj = cuda_core;
     const int cs = attn_cluster_size(ctx, B);
-    const int mma_flat = ctx->attn_v0 || !attn_use_mma(ctx, B) ? 0 : attn_mma_flat_splits(ctx, B);
+    const int slots = ctx->attn_v0 || !ctx->prefilled || !attn_use_mma(ctx, B) ? 0 : attn_balanced_slots(ctx, B);
+    const int mma_flat = ctx->attn_v0 || !attn_use_mma(ctx, B) ? 0 : slots > 0 ? slots : attn_mma_flat_splits(ctx, B);
     const bool mma = attn_use_mma(ctx, B) && (cs <= 8 || mma_flat > 0);
     const bool flat = !ctx->attn_v0 && !mma && attn_flat_now(ctx) && !ctx->attn_cs_force;
     std::string d = "B=" + std::to_string(B) + " projections=" + proj + " attention=" +
                     (ctx->attn_v0 ? std::string("attn_decode_kernel") : mma ? "attn_mma_kernel" : "attn_cluster_kernel") +
-                    (mma_flat > 0 ? " unclustered splits=" + std::to_string(mma_flat)
+                    (slots > 0 ? " unclustered balanced slots=" + std::to_string(slots)
+                     : mma_flat > 0 ? " unclustered splits=" + std::to_string(mma_flat)
                      : flat ? " unclustered splits=" +
                                   std::to_string(std::max(1, std::min({ctx->sms / (B * c.n_kv_heads),
                                                                        (c.max_ctx + 15) / 16, kFlatMaxSplits})))
