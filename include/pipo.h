@@ -344,8 +344,8 @@ PIPO_API size_t pipo_op_gemm_tc_scratch(int32_t mode, int32_t N, int32_t K, int3
  * aligned; K0 and K1 multiples of 64; N, B, splits and the scratch
  * (pipo_op_gemm_tc_scratch(mode, N, K0 + K1, B, splits) bytes, 1024-byte
  * aligned) as pipo_op_gemm_tc.  B <= 32 with one segment or one joint norm
- * runs the converter warps inside the GEMM when B is 16 or 32; every other
- * case prepares the bf16 operand in a separate pass first.  EINVAL for bad
+ * runs the converter warps inside the GEMM; every other case prepares the
+ * bf16 operand in a separate pass first.  EINVAL for bad
  * shapes, alignment, gain combinations or a short scratch buffer. */
 PIPO_API pipo_status pipo_op_gemm_tc_norm(int32_t mode, const void *d_W, int32_t N, const float *d_x0, int32_t K0,
                                           const void *d_gamma0, const float *d_x1, int32_t K1, const void *d_gamma1,

@@ -704,12 +704,16 @@ pipo_status launch_gemm_pair(pipo_ctx* ctx, const GemvParams& p, bf16* xb) {
 // Projection on the tensor cores: the fused GEMM, or bf16 activations from
 // prep_bf16_kernel and then the tcgen05 GEMM.  Eligible: bf16 weights,
 // K % 64 == 0, rows >= 128.  x_rows: rows behind each activation
-// pointer (the tensor maps read no further; at least BH for box-sized maps).
+// pointer, at least B (the tensor maps read no further: rows of a box past them
+// arrive as zeros).  The fused form used to ask for BH rows, so that the
+// kernel-level calls with other batches than 16 and 32 took the two-kernel
+// form: gate/up at 4B, B = 24, 29.0 us against 25.1 (back to back, no
+// dependent launch).
 pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int splits_req, int x_rows) {
     if (p.B > 128) return launch_gemm_pair(ctx, p, xb);
     const int ru = p.epi == EPI_SWIGLU ? 2 : 1;
     const int rows = p.N * ru, bn = tc_bn(p.B), tiles = (rows + kTcM - 1) / kTcM, nkb = p.K / kTcBK;
-    const bool fused = tcf_eligible(p) && !tc_prep_forced() && x_rows >= bn && bn <= tc_fused_max_bh();
+    const bool fused = tcf_eligible(p) && !tc_prep_forced() && x_rows >= p.B && bn <= tc_fused_max_bh();
     // PIPO_TC_SWIGLU_SHALLOW=1: the gate/up projection on the two-per-SM ring
     // (in isolation at B = 16: 22.9 us with two K splits against 24.8 us deep)
     static const bool swiglu_shallow = [] {
