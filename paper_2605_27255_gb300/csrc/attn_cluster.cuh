@@ -72,6 +72,10 @@ struct AttnParams {
     const int32_t* n_pos;   // [nseq] entries before this step
     const float* rope;      // [max_ctx][d_h/2][2] (cos, sin)
     float* out;             // [rows][n_q * d_h]
+    // or (tensor-core kernels, when not null) as bf16 hi rows and, out_lo
+    // elements on, lo rows: the prepared operand of the O projection
+    __nv_bfloat16* out_hi;
+    size_t out_lo;
     float scale;            // 1/sqrt(d_h)
     // Rows (grid z) map to sequences: row r is sequence r % nseq at position
     // n_pos[r % nseq] + r / nseq.  A decode step has one row per sequence
@@ -97,6 +101,19 @@ struct AttnParams {
     // tensor) before the dependency wait; stage_max entries fit
     int stage_max;
 };
+
+// Four consecutive outputs at element i of the attention output.
+__device__ __forceinline__ void attn_store4(const AttnParams& p, size_t i, float4 v) {
+    if (p.out_hi) {
+        uint2 h, l;
+        split_bf16x2(v.x, v.y, h.x, l.x);
+        split_bf16x2(v.z, v.w, h.y, l.y);
+        *reinterpret_cast<uint2*>(p.out_hi + i) = h;
+        *reinterpret_cast<uint2*>(p.out_hi + p.out_lo + i) = l;
+    } else {
+        *reinterpret_cast<float4*>(p.out + i) = v;
+    }
+}
 
 // cos/sin of the 8 rotation pairs of lane slice li at position pos
 template <int DH>

@@ -535,8 +535,8 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
             }
         } else if (CS == 1) {
             const float il = 1.0f / L;
-            *reinterpret_cast<float4*>(p.out + (size_t)row * n_q * DH + (size_t)(g * G + hh) * DH + t) =
-                make_float4(Ov.x * il, Ov.y * il, Ov.z * il, Ov.w * il);
+            attn_store4(p, (size_t)row * n_q * DH + (size_t)(g * G + hh) * DH + t,
+                        make_float4(Ov.x * il, Ov.y * il, Ov.z * il, Ov.w * il));
         } else {
             *reinterpret_cast<float4*>(slot + hh * DH + t) = Ov;
             if (t == 0) {
@@ -598,8 +598,8 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
                     }
             }
             const float il = ms[hh * CS];
-            *reinterpret_cast<float4*>(p.out + (size_t)row * n_q * DH + (size_t)(g * G + hh) * DH + t) =
-                make_float4(Ov.x * il, Ov.y * il, Ov.z * il, Ov.w * il);
+            attn_store4(p, (size_t)row * n_q * DH + (size_t)(g * G + hh) * DH + t,
+                        make_float4(Ov.x * il, Ov.y * il, Ov.z * il, Ov.w * il));
         }
         return;
     }
@@ -637,8 +637,8 @@ __global__ void __launch_bounds__(kMmaThreads) attn_mma_kernel(AttnParams p, con
                 Ov.x += v.x * f; Ov.y += v.y * f; Ov.z += v.z * f; Ov.w += v.w * f;
             }
             const float il = 1.0f / L;
-            *reinterpret_cast<float4*>(p.out + (size_t)row * n_q * DH + (size_t)(g * G + hh) * DH + t) =
-                make_float4(Ov.x * il, Ov.y * il, Ov.z * il, Ov.w * il);
+            attn_store4(p, (size_t)row * n_q * DH + (size_t)(g * G + hh) * DH + t,
+                        make_float4(Ov.x * il, Ov.y * il, Ov.z * il, Ov.w * il));
         }
     }
     PIPO_TR(if (threadIdx.x == 0) {

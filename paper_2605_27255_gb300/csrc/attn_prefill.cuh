@@ -325,11 +325,24 @@ __global__ void __launch_bounds__(kPfThreads, 1) attn_prefill_kernel(AttnParams 
         asm volatile("bar.sync %0, 64;" ::"r"(1 + quad) : "memory");
         if (ok && qvalid) {
             const float inv = 1.0f / (lsum[0][r] + lsum[1][r]);
-            float4* out = reinterpret_cast<float4*>(p.out + (size_t)(jq * B + b) * n_q * DH + (size_t)(g * G + r % G) * DH +
-                                                    hf * 64);
+            const size_t out = (size_t)(jq * B + b) * n_q * DH + (size_t)(g * G + r % G) * DH + hf * 64;
+            if (p.out_hi) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-                out[i] = make_float4(o[4 * i] * inv, o[4 * i + 1] * inv, o[4 * i + 2] * inv, o[4 * i + 3] * inv);
+                for (int i = 0; i < 64; i += 8) {
+                    uint4 h, l;
+                    split_bf16x2(o[i] * inv, o[i + 1] * inv, h.x, l.x);
+                    split_bf16x2(o[i + 2] * inv, o[i + 3] * inv, h.y, l.y);
+                    split_bf16x2(o[i + 4] * inv, o[i + 5] * inv, h.z, l.z);
+                    split_bf16x2(o[i + 6] * inv, o[i + 7] * inv, h.w, l.w);
+                    *reinterpret_cast<uint4*>(p.out_hi + out + i) = h;
+                    *reinterpret_cast<uint4*>(p.out_hi + p.out_lo + out + i) = l;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 64; i += 4)
+                    *reinterpret_cast<float4*>(p.out + out + i) =
+                        make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
+            }
         }
     }
     tc_fence_before();

@@ -44,7 +44,11 @@ void* k_pick_tcv(int bh, bool deep, bool fused) {
 
 void* k_pick_pair() { return reinterpret_cast<void*>(&gemm_pair_kernel<kPairN>); }
 
-void* k_pick_prep_bf16() { return reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16>); }
+void* k_pick_prep_bf16(int threads) {
+    return threads == 128   ? reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16, 128>)
+           : threads == 256 ? reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16, 256>)
+                            : reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16, kPrepThreads>);
+}
 
 cudaError_t k_error_word_tc(const unsigned** p) { return unit_error_word(p); }
 cudaError_t k_take_error_tc(unsigned* code, unsigned* info) { return take_unit_error(code, info); }

@@ -52,6 +52,14 @@ struct GemvParams {
     float eps;
     unsigned long long* zero_ptr;  // zeroed by block 0 before anything else (or nullptr)
     int zero_n;
+    // tensor-core projections with a prepared operand: xready, the input as bf16
+    // hi and lo rows already (written by the kernel that produced it; no
+    // preparation pass); EPI_SWIGLU with yb: the outputs as bf16 hi rows
+    // [b][N] and, yb_lo elements on, lo rows in place of fp32 (the operand of
+    // the projection after)
+    void* xready;
+    void* yb;
+    size_t yb_lo;
     // L2 warm-up of the next attention's cached pages (streaming GEMV, a
     // decode step's QKV projection; pf_k == nullptr: none).  Before its
     // dependency wait the kernel prefetches into L2 the key and value pages
@@ -143,6 +151,15 @@ template <typename T> __device__ __forceinline__ float ldw(const void* p, size_t
 template <typename T> __device__ __forceinline__ T from_f(float v);
 template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
+
+// x as bf16 part hi = bf16(x) and remainder lo = bf16(x - hi), two values packed
+__device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    const float2 f = __bfloat1622float2(h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - f.x, x1 - f.y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
 
 __device__ __forceinline__ float silu(float x) { return x / (1.0f + expf(-x)); }
 
@@ -253,26 +270,45 @@ __device__ __forceinline__ size_t kv_off(const KVView& kv, int b, int pos, int g
 // value, before the chunk's attention reads them (row r is sequence r % nseq
 // at position n_pos[r % nseq] + r / nseq).  Rotate-half with the fp32
 // cos/sin table the attention kernels use ([max_ctx][d_h/2][2]), rounded to
-// the cache type.  grid (rows, n_kv), DH/2 threads.
+// the cache type.  grid rows; a thread takes four rotation pairs of a kv head.
+// Bound by its n_kv * d_h * (8 + 2 sizeof(T)) bytes per row; one CTA of d_h / 2
+// threads per row and head took 16.7 us at 1792 rows (8 heads of 128), one CTA
+// per row 6.0.
+constexpr int kAppendThreads = 128;
+template <typename T>
+__device__ __forceinline__ void st4(T* p, float4 v) {
+    if constexpr (sizeof(T) == 4) *reinterpret_cast<float4*>(p) = v;
+    else {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(p) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    }
+}
 template <typename T, int DH>
-__global__ void append_rows_kernel(const float* __restrict__ qkv, int ld_qkv, int n_q, KVView kv,
-                                   const int32_t* __restrict__ n_pos, int nseq, const float* __restrict__ rope) {
+__global__ void __launch_bounds__(kAppendThreads)
+    append_rows_kernel(const float* __restrict__ qkv, int ld_qkv, int n_q, KVView kv, const int32_t* __restrict__ n_pos,
+                       int nseq, const float* __restrict__ rope) {
     pdl_launch();
     pdl_wait();
-    const int row = blockIdx.x, g = blockIdx.y, i = threadIdx.x;
-    const int b = row % nseq;
+    const int row = blockIdx.x, b = row % nseq;
     const int pos = n_pos[b] + row / nseq;
-    const float* k = qkv + (size_t)row * ld_qkv + (size_t)(n_q + g) * DH;
-    const float* v = qkv + (size_t)row * ld_qkv + (size_t)(n_q + kv.n_kv + g) * DH;
-    const float c = rope[((size_t)pos * (DH / 2) + i) * 2], s = rope[((size_t)pos * (DH / 2) + i) * 2 + 1];
-    const float a = k[i], bb = k[i + DH / 2];
-    const size_t off = kv_off<T, DH>(kv, b, pos, g);
-    T* K = static_cast<T*>(kv.K) + off;
-    T* V = static_cast<T*>(kv.V) + off;
-    K[i] = from_f<T>(a * c - bb * s);
-    K[i + DH / 2] = from_f<T>(bb * c + a * s);
-    V[i] = from_f<T>(v[i]);
-    V[i + DH / 2] = from_f<T>(v[i + DH / 2]);
+    const float* base = qkv + (size_t)row * ld_qkv + (size_t)n_q * DH;
+    const float4* rp = reinterpret_cast<const float4*>(rope + (size_t)pos * DH);  // cos, sin, cos, sin
+    for (int it = threadIdx.x; it < kv.n_kv * (DH / 8); it += kAppendThreads) {
+        const int g = it / (DH / 8), i = (it % (DH / 8)) * 4;
+        const float4* k = reinterpret_cast<const float4*>(base + (size_t)g * DH + i);
+        const float4* v = reinterpret_cast<const float4*>(base + (size_t)(kv.n_kv + g) * DH + i);
+        const float4 r0 = rp[i / 2], r1 = rp[i / 2 + 1], ka = k[0], kb = k[DH / 8], va = v[0], vb = v[DH / 8];
+        const size_t off = kv_off<T, DH>(kv, b, pos, g) + i;
+        T* K = static_cast<T*>(kv.K) + off;
+        T* V = static_cast<T*>(kv.V) + off;
+        st4(K, make_float4(ka.x * r0.x - kb.x * r0.y, ka.y * r0.z - kb.y * r0.w, ka.z * r1.x - kb.z * r1.y,
+                           ka.w * r1.z - kb.w * r1.w));
+        st4(K + DH / 2, make_float4(kb.x * r0.x + ka.x * r0.y, kb.y * r0.z + ka.y * r0.w, kb.z * r1.x + ka.z * r1.y,
+                                    kb.w * r1.z + ka.w * r1.w));
+        st4(V, va);
+        st4(V + DH / 2, vb);
+    }
 }
 
 // RoPE on q and k (rotate-half, angle = pos * theta^(-2i/d) in double), then

@@ -128,6 +128,7 @@ struct pipo_ctx {
     unsigned long long* am = nullptr;  // [2][max_batch]
     // tensor-core projections (bf16, batch >= tc_min_b)
     bf16* tc_xb = nullptr;          // [2 * tc_bn_max][tc_kmax] bf16 activations (hi rows, lo rows)
+    bf16* tc_act = nullptr;         // [2 * tc_bn_max][ffn] the same for the down projection, written by gate/up
     int tc_kmax = 0, tc_bn_max = 0;
     int act_rows = 0;               // rows of the fp32 activation buffers (>= the batch width BH)
     bool tc_shallow = false;        // this step's projections: two-per-SM ring (room for a co-resident neighbour)
@@ -519,6 +520,22 @@ pipo_status make_tmap_y(pipo_ctx* ctx, CUtensorMap* tm, float* base, int N, int 
     return PIPO_OK;
 }
 
+// The same for bf16 outputs.
+pipo_status make_tmap_yb(pipo_ctx* ctx, CUtensorMap* tm, bf16* base, int N, int ld, int rows, int box_n, int box_rows) {
+    TRY(load_encoder(ctx));
+    if (!base || reinterpret_cast<uintptr_t>(base) % 16 != 0 || ld % 8 != 0 || N < 1 || rows < 1)
+        return fail(ctx, PIPO_EINVAL, "bf16 output tensor map: base %% 16, ld %% 8 required");
+    const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)box_n, (cuuint32_t)box_rows};
+    const cuuint32_t es[2] = {1, 1};
+    const CUresult r = g_encode_tiled(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, es,
+                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, PIPO_ECUDA, "cuTensorMapEncodeTiled (bf16 outputs): error %d", (int)r);
+    return PIPO_OK;
+}
+
 // rows of the activation buffers behind a batch of B: the box height up to 32
 int tc_bn(int B) { return B <= 16 ? 16 : B <= 32 ? 32 : B <= 64 ? 64 : B <= 128 ? 128 : B; }
 
@@ -682,20 +699,30 @@ pipo_status launch_gemm_pair(pipo_ctx* ctx, const GemvParams& p, bf16* xb) {
     q.tiles_n = (p.B + kPairN - 1) / kPairN;
     q.tiles = (rows + kPairM - 1) / kPairM * q.tiles_n;
     const int pairs = std::min(q.tiles, std::max(1, pair_max_clusters()));
-    CUtensorMap tmW, tmX, tmY;
+    if (p.xready) xb = static_cast<bf16*>(p.xready);
+    CUtensorMap tmW, tmX, tmY, tmY2;
     TRY(make_tmap(ctx, &tmW, p.W, p.K, rows, kTcM));
     TRY(make_tmap(ctx, &tmX, xb, p.K, 2 * p.B, kPairN / 2));
-    TRY(make_tmap_y(ctx, &tmY, p.y, p.N, p.ldy, p.B, 32 / ru, kPairOutN));
-    {
+    if (p.yb && ru == 2) {
+        bf16* yb = static_cast<bf16*>(p.yb);
+        q.split_out = 1;
+        TRY(make_tmap_yb(ctx, &tmY, yb, p.N, p.ldy, p.B, 64, kPairOutN));
+        TRY(make_tmap_yb(ctx, &tmY2, yb + p.yb_lo, p.N, p.ldy, p.B, 64, kPairOutN));
+    } else {
+        TRY(make_tmap_y(ctx, &tmY, p.y, p.N, p.ldy, p.B, 32 / ru, kPairOutN));
+        tmY2 = tmY;
+    }
+    if (!p.xready) {
         GemvParams pp = p;
         int bh = p.B;
         void* args[] = {&pp, &xb, &bh};
         ctx->prof_kind = 2;
         ctx->prof_bytes = 0.0;
         ctx->launch_prep = true;
-        TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16()), dim3(p.B), dim3(kPrepThreads), 0, args));
+        const int nt = prep_threads(p.K, p.B);
+        TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16(nt)), dim3(p.B), dim3(nt), 0, args));
     }
-    void* args[] = {&tmW, &tmX, &tmY, &q};
+    void* args[] = {&tmW, &tmX, &tmY, &tmY2, &q};
     ctx->prof_kind = 0;
     ctx->prof_bytes = (double)rows * p.K * 2;
     return launch_ex(ctx, k_pick_pair(), dim3(2 * pairs), dim3(kPairThreads), kPairSmem, args, 2);
@@ -727,6 +754,7 @@ pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int spl
     tp.rows = rows; tp.K = p.K; tp.B = p.B; tp.ru = ru; tp.epi = p.epi;
     tp.y = p.y; tp.ldy = p.ldy; tp.bias = p.bias; tp.am = p.am; tp.dbg = p.dbg; tp.ld_dbg = p.ld_dbg;
     tp.splits = plan.splits;
+    if (p.xready) xb = static_cast<bf16*>(p.xready);
     if (fused) {
         CUtensorMap tmW, tmX0, tmX1;
         TRY(make_tmap(ctx, &tmW, p.W, p.K, rows, kTcM));
@@ -753,14 +781,14 @@ pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int spl
     CUtensorMap tmW, tmX;
     TRY(make_tmap(ctx, &tmW, p.W, p.K, rows, kTcM));
     TRY(make_tmap(ctx, &tmX, xb, p.K, 2 * bn, 2 * bn));
-    {
+    if (!p.xready) {
         GemvParams pp = p;
         int bh = bn;
         void* args[] = {&pp, &xb, &bh};
         ctx->prof_kind = 2;
         ctx->prof_bytes = 0.0;
         ctx->launch_prep = true;
-        TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16()), dim3(bn), dim3(kPrepThreads), 0,
+        TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16(kPrepThreads)), dim3(bn), dim3(kPrepThreads), 0,
                       args));
     }
     void* args[] = {&tmW, &tmX, &tp};
@@ -940,7 +968,7 @@ cudaError_t set_carveouts(bool bf) {
             for (bool deep : {false, true})
                 for (bool fused : {false, true}) fns.push_back(pick_tcv(bn, deep, fused));
         fns.push_back(k_pick_pair());
-        fns.push_back(reinterpret_cast<const void*>(k_pick_prep_bf16()));
+        for (int n : {128, 256, kPrepThreads}) fns.push_back(reinterpret_cast<const void*>(k_pick_prep_bf16(n)));
         for (int g : {1, 2, 4})
             for (bool deep : {false, true}) fns.push_back(attnm_pick(g, deep));
     }
@@ -1187,11 +1215,29 @@ bool prefill_tiles(const pipo_ctx* ctx, int R) {
     return R >= 64 && R / ctx->B >= 8;
 }
 
+// Rows the bf16 hi part of a projection's prepared operand takes before its lo
+// part, or 0 when the projection prepares nothing (GEMV, fused form).  Batches
+// of more than 32 rows: the producers of such an operand write it themselves.
+int tc_prepared_rows(const pipo_ctx* ctx, int N, int K, int R) {
+    GemvParams p{};
+    p.N = N; p.K = K; p.B = R; p.epi = EPI_STORE;
+    if (R <= 32 || !tc_eligible(ctx, p) || (R <= 128 && tc_bn(R) <= tc_fused_max_bh())) return 0;
+    return R > 128 ? R : tc_bn(R);
+}
+
 // One decoder block on the residual stream xr (pre-norm attention + SwiGLU).
 pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, float* xr) {
     const pipo_config& c = ctx->cfg;
     const int H = c.hidden, DH = c.head_dim, qd = c.n_q_heads * DH, kd = c.n_kv_heads * DH, rows = qd + 2 * kd;
     const bool bf = c.dtype == 1;
+    const int R_blk = ctx->rows > 0 ? ctx->rows : ctx->B;
+    // the attention and (on the CTA-pair GEMM, whose outputs leave as tiles; the
+    // narrow kernels' two-byte stores cost more than the preparation, 128 rows
+    // 14.4 -> 16.3 ms) the gate/up projection write the next projection's
+    // operand themselves where that one would prepare it: a launch less each
+    int o_hi = tc_prepared_rows(ctx, H, qd, R_blk);
+    const int act_hi = ctx->tc_act && R_blk > 128 && tc_prepared_rows(ctx, 2 * c.ffn, H, R_blk) > 0
+                           ? tc_prepared_rows(ctx, H, c.ffn, R_blk) : 0;
     // RMSNorm -> fused QKV projection
     GemvParams p = gemv_base(ctx, bw.Wqkv, rows, EPI_STORE, ctx->qkv, rows);
     p.seg[0] = act_seg(xr, H, H, bw.attn_norm);
@@ -1222,7 +1268,7 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
             const float* rope = ctx->rope;
             void* args[] = {(void*)&qkv, &ld, &nq, &kv, (void*)&np, &nseq, (void*)&rope};
             void* fn = k_pick_append_rows(bf, DH);
-            TRY(launch_ex(ctx, fn, dim3(R, c.n_kv_heads), dim3(DH / 2), 0, args));
+            TRY(launch_ex(ctx, fn, dim3(R), dim3(kAppendThreads), 0, args));
         }
         // outside a graph a launch or two earlier may still write the lengths
         // and entries that the attention reads before its dependency wait
@@ -1248,6 +1294,21 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
         ap.no_append = chunk ? 1 : 0;
         void* args[] = {&ap};
         const int cs = attn_cluster_size(ctx, R);
+        const bool mma = (chunk && prefill_tiles(ctx, R)) ||
+                         (attn_use_mma(ctx, R) &&
+                          (cs <= 8 || (!chunk && (attn_balanced_slots(ctx, R) > 0 || attn_mma_flat_splits(ctx, R) > 0))));
+        if (!mma) o_hi = 0;  // the other attention kernels write fp32
+        // a tile attention that leaves SMs idle keeps the preparation: without
+        // it the O projection's CTAs settle, two to an SM, on the SMs that the
+        // attention does not use (4 x 1024 tokens, 32 CTAs: 14.48 against 14.84 ms)
+        if (chunk && prefill_tiles(ctx, R)) {
+            const int TP = kPfVec / (c.n_q_heads / c.n_kv_heads), C = R / ctx->B;
+            if ((long long)((C + TP - 1) / TP) * c.n_kv_heads * ctx->B < ctx->sms) o_hi = 0;
+        }
+        if (o_hi > 0) {
+            ap.out_hi = ctx->tc_xb;
+            ap.out_lo = (size_t)o_hi * qd;
+        }
         const int G = c.n_q_heads / c.n_kv_heads;
         if (chunk && prefill_tiles(ctx, R)) {
             // causal tiles: the positions of a tile share every key and value they read
@@ -1304,6 +1365,7 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
                           cs));
         }
     } else {
+    o_hi = 0;
     // RoPE + KV append
     {
         const float* qkv = ctx->qkv;
@@ -1335,16 +1397,22 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
     p = gemv_base(ctx, bw.Wo, H, EPI_RESADD, xr, H);
     p.seg[0] = act_seg(ctx->attn, qd, qd);
     p.K = qd;
+    if (o_hi > 0) p.xready = ctx->tc_xb;
     TRY(launch_gemv(ctx, p));
     // RMSNorm -> gate|up -> SwiGLU
     p = gemv_base(ctx, bw.Wgu, c.ffn, EPI_SWIGLU, ctx->act, c.ffn);
     p.seg[0] = act_seg(xr, H, H, bw.ffn_norm);
     p.K = H;
+    if (act_hi > 0) {
+        p.yb = ctx->tc_act;
+        p.yb_lo = (size_t)act_hi * c.ffn;
+    }
     TRY(launch_gemv(ctx, p));
     // down projection + residual
     p = gemv_base(ctx, bw.Wdown, H, EPI_RESADD, xr, H);
     p.seg[0] = act_seg(ctx->act, c.ffn, c.ffn);
     p.K = c.ffn;
+    if (act_hi > 0) p.xready = ctx->tc_act;
     TRY(launch_gemv(ctx, p));
     return PIPO_OK;
 }
@@ -1968,6 +2036,7 @@ pipo_status pipo_init(const pipo_config* cfg, const pipo_weights* w, pipo_ctx** 
             ctx->tc_bn_max = tc_bn(std::max(std::min(MB, 128), ctx->prefill_rows));
             ctx->tc_kmax = std::max({2 * (int)H, qd, c.ffn});
             TRY(dalloc(ctx, &ctx->tc_xb, (size_t)2 * ctx->tc_bn_max * ctx->tc_kmax * 2));
+            if (ctx->tc_bn_max > 128) TRY(dalloc(ctx, &ctx->tc_act, (size_t)2 * ctx->tc_bn_max * c.ffn * 2));
         }
         TRY(dalloc(ctx, &ctx->pending, (size_t)MB * 2 * 4));
         TRY(dalloc(ctx, &ctx->n_pos, (size_t)MB * 4));

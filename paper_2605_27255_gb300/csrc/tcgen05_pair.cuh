@@ -60,6 +60,7 @@ struct PairParams {
     int K, B;          // inputs, positions
     int ru, epi;       // as TcParams
     const void* bias;  // bf16 [rows]
+    int split_out;     // ru == 2: outputs as bf16 hi (tmY) and lo (tmY2) instead of fp32 (tmY)
     int tiles_n;       // position tiles
     int tiles;         // weight tiles * position tiles
 };
@@ -114,6 +115,13 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// a store that joins the bulk group of the tma_store_2d after it
+__device__ __forceinline__ void tma_store_2d_more(const CUtensorMap* tm, int x, int y, const void* src) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tm), "r"(x), "r"(y),
+                 "r"(smem_u32(src))
+                 : "memory");
+}
+
 // shared -> global 2-D tensor store (or fp32 add) of the box at element
 // coordinates (x, y); parts outside the tensor are left out
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, int x, int y, const void* src, bool add) {
@@ -133,7 +141,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, int x, int y
 template <int NT>
 __global__ void __launch_bounds__(kPairThreads, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-                     const __grid_constant__ CUtensorMap tmY, PairParams p) {
+                     const __grid_constant__ CUtensorMap tmY, const __grid_constant__ CUtensorMap tmY2, PairParams p) {
     extern __shared__ __align__(1024) unsigned char tp_smem_raw[];
     __shared__ uint32_t tmem_base;
     constexpr int ST = kPairStages, SB = kPairStageBytes;
@@ -270,15 +278,15 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         float* mine = out_s + (warp - 4) * 2 * kPairOutN * 32;
         pdl_wait();
         int sc = 0, oc = 0;  // segments, output stores so far
-        bool ok = true;
-        for (int t = cid; t < p.tiles && ok; t += ncl) {
+        bool ok = true;  // once a wait has given up, the tiles run through without waiting (the barriers stay matched)
+        for (int t = cid; t < p.tiles; t += ncl) {
             const int m = t / p.tiles_n, n = t % p.tiles_n;
             float acc[nc];
 #pragma unroll
             for (int j = 0; j < nc; ++j) acc[j] = 0.f;
             for (int i0 = 0; i0 < nk; i0 += kPairSeg, ++sc) {
                 const int buf = sc & 1;
-                if (!mbar_wait(accf + buf, (uint32_t)((sc >> 1) & 1), 35, sc)) { ok = false; break; }
+                ok = ok && mbar_wait(accf + buf, (uint32_t)((sc >> 1) & 1), 35, sc);
                 __syncwarp();
                 tc_fence_after();
                 // 64 columns per wait: with 16 the loads' latency, eight times
@@ -294,10 +302,42 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive_at(acce_lead + 8 * buf);
             }
-            if (!ok) break;
             // outputs through the warp's two buffers [kPairOutN][32 / ru] and
             // tensor stores, which overlap the next tile (its MMAs wait for
             // these warps after two segments)
+            if (p.split_out) {
+                // SwiGLU as the next projection's operand: the four warps of
+                // these positions share a tile of 64 outputs (bf16 hi and lo, rows
+                // of 128 bytes; stores of 32-byte rows, a warp's own 16 outputs,
+                // cost 29 us of 210 at 1792 rows)
+                const int b0 = n * NT + ch, u0 = (m * kPairM + half * 128) / 2, id = 1 + (warp - 4) / 4;
+                __nv_bfloat16* shared = reinterpret_cast<__nv_bfloat16*>(out_s) + (warp - 4) / 4 * (2 * 2 * kPairOutN * 64);
+                const bool odd = lane & 1;
+#pragma unroll
+                for (int c0 = 0; c0 < nc; c0 += kPairOutN)
+                    if (b0 + c0 < p.B && 2 * u0 < p.rows) {
+                        __nv_bfloat16* hi = shared + (oc++ & 1) * 2 * kPairOutN * 64;
+                        if (quad == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
+#pragma unroll
+                        for (int j = 0; j < kPairOutN; j += 2) {
+                            const float v0 = acc[c0 + j], v1 = acc[c0 + j + 1];
+                            const float o = __shfl_xor_sync(0xffffffffu, odd ? v0 : v1, 1);
+                            const float a = silu(odd ? o : v0) * (odd ? v1 : o);
+                            const __nv_bfloat16 h = __float2bfloat16_rn(a);
+                            const int at = (j + odd) * 64 + quad * 16 + (lane >> 1);
+                            hi[at] = h;
+                            hi[kPairOutN * 64 + at] = __float2bfloat16_rn(a - __bfloat162float(h));
+                        }
+                        fence_proxy_async();
+                        asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory");
+                        if (quad == 0 && lane == 0) {
+                            tma_store_2d_more(&tmY2, u0, b0 + c0, hi + kPairOutN * 64);
+                            tma_store_2d(&tmY, u0, b0 + c0, hi, false);
+                        }
+                    }
+                continue;
+            }
             const int b0 = n * NT + ch, ru = p.ru, row0 = m * kPairM + half * 128 + quad * 32, row = row0 + lane;
             const float bias = p.epi == EPI_BIAS && row < p.rows
                                    ? __bfloat162float(static_cast<const __nv_bfloat16*>(p.bias)[row]) : 0.f;
