@@ -515,9 +515,15 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // gsm: K elements of type T for the gains.  Same split layout as stage_input_fast.
 // yres (EPI_RESADD, or nullptr): [units][NB] receives y of units [u0, u0 +
 // units) of sequences b0 .. b0 + nb - 1, loaded while the input copies fly.
+// One norm over the whole input (a single segment, or a joint norm): the
+// staged values are gain * x and rs[bb] receives the factor 1 / rms, which the
+// caller multiplies into the finished sums; it is summed up after the last
+// barrier, under the weight loop, instead of between two more of them.  rs = 1
+// otherwise.
 template <typename T, int NB>
 __device__ __forceinline__ void stage_input_async(const GemvParams& p, float* xs, T* gsm, int b0, int nb,
-                                                  float (*yres)[NB] = nullptr, int u0 = 0, int units = 0) {
+                                                  float (&rs)[NB], float (*yres)[NB] = nullptr, int u0 = 0,
+                                                  int units = 0) {
     __shared__ float red_ss[32][NB][2];
     __shared__ float rstd_s[NB][2];
     const int K = p.K, K0q = p.seg[0].K / 4;
@@ -567,7 +573,35 @@ __device__ __forceinline__ void stage_input_async(const GemvParams& p, float* xs
     if (yres && tid < units * nb) yres[tid / nb][tid % nb] = yv;  // units * nb <= the block's threads
     cp_async_wait_all();
     __syncthreads();
+#pragma unroll
+    for (int bb = 0; bb < NB; ++bb) rs[bb] = 1.f;
     if (!norm0 && !norm1) return;
+    if (p.nseg == 1 || p.joint_norm) {
+        float sq[NB];
+#pragma unroll
+        for (int bb = 0; bb < NB; ++bb) sq[bb] = 0.f;
+        for (int q = tid; q < K / 4; q += nt) {
+            const float4 gm = ld4<T>(gsm, (size_t)q * 4);
+#pragma unroll
+            for (int bb = 0; bb < NB; ++bb) {
+                float4* xp = reinterpret_cast<float4*>(xs + bb * K + xidx(q));
+                float4 v = *xp;
+                sq[bb] += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+                v.x *= gm.x; v.y *= gm.y; v.z *= gm.z; v.w *= gm.w;
+                *xp = v;
+            }
+        }
+#pragma unroll
+        for (int bb = 0; bb < NB; ++bb) {
+            const float a = warp_sum(sq[bb]);
+            if (lane == 0) red_ss[warp][bb][0] = a;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int bb = 0; bb < NB; ++bb)
+            rs[bb] = 1.0f / sqrtf(warp_sum(lane < nt / 32 ? red_ss[lane][bb][0] : 0.f) / (float)K + p.eps);
+        return;
+    }
     // sums of squares per sequence and norm group
     const int K4 = K / 4;
     float ss[NB][2];
@@ -666,7 +700,8 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
         }
         const bool ypre_on = p.epi == EPI_RESADD && u1 - u0 <= kYpreUnits;
         __syncthreads();
-        stage_input_async<T, NB>(p, xs, reinterpret_cast<T*>(xs + NB * K), b0, nb, ypre_on ? ypre_s : nullptr, u0,
+        float rs[NB];
+        stage_input_async<T, NB>(p, xs, reinterpret_cast<T*>(xs + NB * K), b0, nb, rs, ypre_on ? ypre_s : nullptr, u0,
                                  u1 - u0);
 
         float best_v[NB];
@@ -712,7 +747,7 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
                         const int r = crow % RU;
 #pragma unroll
                         for (int bb = 0; bb < NB; ++bb) {
-                            const float t = warp_sum(acc[bb]);
+                            const float t = warp_sum(acc[bb]) * rs[bb];
                             acc[bb] = 0.f;
 #pragma unroll
                             for (int rr = 0; rr < RU; ++rr)
@@ -757,7 +792,7 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
             float a[RU][NB];
 #pragma unroll
             for (int bb = 0; bb < NB; ++bb) {
-                const float t = warp_sum(acc[bb]);
+                const float t = warp_sum(acc[bb]) * rs[bb];
 #pragma unroll
                 for (int rr = 0; rr < RU; ++rr) a[rr][bb] = part[rr][bb] + ((rr == r && cj > 0) ? t : 0.f);
             }
