@@ -44,6 +44,11 @@ void* k_pick_tcv(int bh, bool deep, bool fused) {
 
 void* k_pick_pair() { return reinterpret_cast<void*>(&gemm_pair_kernel<kPairN>); }
 
+void* k_pick_pair_mid(int nt) {
+    return nt == 64 ? reinterpret_cast<void*>(&gemm_pair_mid_kernel<64>)
+                    : reinterpret_cast<void*>(&gemm_pair_mid_kernel<kPairMidN>);
+}
+
 void* k_pick_prep_bf16(int threads) {
     return threads == 128   ? reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16, 128>)
            : threads == 256 ? reinterpret_cast<void*>(&prep_bf16_kernel<__nv_bfloat16, 256>)

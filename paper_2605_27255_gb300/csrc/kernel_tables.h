@@ -19,6 +19,7 @@ void* k_pick_stream_f32(int nb, int ru, bool rows);
 // k_tc.cu: the tcgen05 projections
 void* k_pick_tcv(int bh, bool deep, bool fused);    // gemm_tcf_kernel (fused) / gemm_tc_kernel
 void* k_pick_pair();                                // gemm_pair_kernel
+void* k_pick_pair_mid(int nt);                      // gemm_pair_mid_kernel<64 or 128>
 void* k_pick_prep_bf16(int threads);                // prep_bf16_kernel<bf16, threads>
 cudaError_t k_error_word_tc(const unsigned** p);      // device address of the unit's error word
 cudaError_t k_take_error_tc(unsigned* code, unsigned* info);

@@ -135,6 +135,7 @@ struct pipo_ctx {
     int tc_min_b = 2;               // measured: a tie with the CUDA-core GEMV at B = 1, far ahead from B = 4
     int attn_mma_min_b = 1;         // smallest batch on the tensor-core attention (PIPO_ATTN_MMA_MIN_BATCH)
     int tc_splits = 0;              // forced K splits (0: automatic)
+    bool op_call = false;           // settings of a kernel-level call, not a model's context
 
     int32_t *pending = nullptr, *n_pos = nullptr, *out_tokens = nullptr, *out_nacc = nullptr;
     // mapped host memory, written by the kernel that ends a step: tokens
@@ -447,7 +448,14 @@ cudaError_t set_smem_attrs(bool bf) {
                                                                  : cudaClusterSchedulingPolicyLoadBalancing);
                     if (e != cudaSuccess) return e;
                 }
-    if (bf) return cudaFuncSetAttribute(k_pick_pair(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+    if (bf) {
+        for (int nt : {64, kPairMidN}) {
+            const cudaError_t e = cudaFuncSetAttribute(k_pick_pair_mid(nt), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)pair_mid_smem(nt));
+            if (e != cudaSuccess) return e;
+        }
+        return cudaFuncSetAttribute(k_pick_pair(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+    }
     return cudaSuccess;
 }
 
@@ -659,34 +667,61 @@ int tc_fused_max_bh() {
     return v;
 }
 
-// CTA pairs of the CTA-pair GEMM that can be resident at once on the current
-// device (cached).
-int pair_max_clusters() {
+// Clusters of 2 * splits CTAs of a CTA-pair GEMM that can be resident at once on
+// the current device (cached).
+int pair_clusters(void* fn, int splits, size_t smem) {
     static std::mutex mu;
-    static std::map<int, int> cache;
+    static std::map<std::pair<void*, int>, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 0; }
     std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(dev);
+    const auto key = std::make_pair(fn, dev * 16 + splits);
+    auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(2);
+    lc.gridDim = dim3(2 * splits);
     lc.blockDim = dim3(kPairThreads);
-    lc.dynamicSmemBytes = kPairSmem;
+    lc.dynamicSmemBytes = smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.x = 2 * splits;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_pick_pair(), &lc) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &lc) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
     }
-    cache[dev] = n;
+    cache[key] = n;
     return n;
+}
+int pair_max_clusters() { return pair_clusters(k_pick_pair(), 1, kPairSmem); }
+
+// Projection of 33 .. 64 (nt = 64) or 65 .. 128 rows (nt = 128) on CTA pairs,
+// from the prepared operand xb.
+pipo_status launch_gemm_pair_mid(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int nt, int splits_req) {
+    void* fn = k_pick_pair_mid(nt);
+    const size_t smem = pair_mid_smem(nt);
+    const int ru = p.epi == EPI_SWIGLU ? 2 : 1, rows = p.N * ru, nkb = p.K / kTcBK;
+    PairMidParams q{};
+    q.rows = rows; q.K = p.K; q.B = p.B; q.ru = ru; q.epi = p.epi; q.y = p.y; q.ldy = p.ldy; q.bias = p.bias;
+    q.tiles = (rows + kPairM - 1) / kPairM;
+    // K splits while whole clusters of them are resident, kTcMinKb K blocks each
+    int S = splits_req > 0 ? std::min({splits_req, nkb, kPairMaxSplits})
+                           : std::max(1, std::min({ctx->sms / 2 / q.tiles, nkb / kTcMinKb, kPairMaxSplits}));
+    if (splits_req <= 0)
+        while (S > 1 && pair_clusters(fn, S, smem) < q.tiles) --S;
+    q.splits = S;
+    const int clusters = S > 1 ? q.tiles : std::min(q.tiles, std::max(1, pair_clusters(fn, 1, smem)));
+    CUtensorMap tmW, tmX;
+    TRY(make_tmap(ctx, &tmW, p.W, p.K, rows, kTcM));
+    TRY(make_tmap(ctx, &tmX, xb, p.K, 2 * nt, nt));
+    void* args[] = {&tmW, &tmX, &q};
+    ctx->prof_kind = 0;
+    ctx->prof_bytes = (double)rows * p.K * 2;
+    return launch_ex(ctx, fn, dim3(clusters * 2 * S), dim3(kPairThreads), smem, args, 2 * S);
 }
 
 // Projection of a prefill chunk of more than 128 rows: bf16 hi and lo rows
@@ -791,6 +826,13 @@ pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int spl
         TRY(launch_ex(ctx, reinterpret_cast<const void*>(k_pick_prep_bf16(kPrepThreads)), dim3(bn), dim3(kPrepThreads), 0,
                       args));
     }
+    // CTA pairs from 33 rows on.  Alone (graph of calls, preparation included, us,
+    // one CTA / pairs, 4B shapes) 128 rows QKV 23.2 / 20.2, O 18.8 / 16.4, gate/up
+    // 35.4 / 29.4, down 28.1 / 24.9; 64 rows 15.3 / 17.5, 12.7 / 14.4, 25.8 / 25.8,
+    // 19.4 / 22.8; but inside a step, where the pairs' start overlaps the launch
+    // before, 64 rows are ahead too (six 4B-wide layers 1.147 -> 1.121 ms)
+    if (p.epi != EPI_ARGMAX && (bn == kPairMidN || (bn == 64 && !ctx->op_call)))
+        return launch_gemm_pair_mid(ctx, p, xb, bn, splits_req);
     void* args[] = {&tmW, &tmX, &tp};
     ctx->prof_kind = 0;
     ctx->prof_bytes = (double)rows * p.K * 2;
@@ -967,7 +1009,7 @@ cudaError_t set_carveouts(bool bf) {
         for (int bn : {16, 32, 64, 128})
             for (bool deep : {false, true})
                 for (bool fused : {false, true}) fns.push_back(pick_tcv(bn, deep, fused));
-        fns.push_back(k_pick_pair());
+        for (void* f : {k_pick_pair(), k_pick_pair_mid(64), k_pick_pair_mid(kPairMidN)}) fns.push_back(f);
         for (int n : {128, 256, kPrepThreads}) fns.push_back(reinterpret_cast<const void*>(k_pick_prep_bf16(n)));
         for (int g : {1, 2, 4})
             for (bool deep : {false, true}) fns.push_back(attnm_pick(g, deep));
@@ -2592,6 +2634,7 @@ pipo_status op_setup(pipo_ctx& op, int32_t dtype, void* stream) {
     }
     op.stream = static_cast<cudaStream_t>(stream);
     op.pdl = false;
+    op.op_call = true;
     return PIPO_OK;
 }
 
@@ -2941,7 +2984,8 @@ pipo_status pipo_describe_step(const pipo_ctx* ctx, char* h_buf, size_t cap) {
     const std::string cuda_core = B <= 4 ? "gemv_rows_kernel" : "gemv_kernel";
     const bool fused = !tc_prep_forced() && tc_bn(B) <= tc_fused_max_bh();
     const std::string tck = fused ? "gemm_tcf_kernel<" + std::to_string(tc_bn(B)) + ">"
-                                  : "gemm_tc_kernel<" + std::to_string(tc_bn(B)) + ">+prep_bf16_kernel";
+                                  : (B > 32 && B <= 128 ? "gemm_pair_mid_kernel<" : "gemm_tc_kernel<") + std::to_string(tc_bn(B)) +
+                                        ">+prep_bf16_kernel";
     if (n_tc == 4) proj = tck + " (tcgen05)";
     else if (n_tc > 0) proj = tck + " (tcgen05; " + std::to_string(4 - n_tc) + " of 4 block projections on " +
                               cuda_core + ")";

@@ -120,8 +120,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 64 consecutive fp32 columns of this thread's TMEM lane, one wait
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
+// twice 32 consecutive fp32 columns of this thread's TMEM lane, `gap` apart, one wait
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64], uint32_t gap = 32) {
     uint32_t r[64];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -136,7 +136,7 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
               "=r"(r[32 * h + 20]), "=r"(r[32 * h + 21]), "=r"(r[32 * h + 22]), "=r"(r[32 * h + 23]),
               "=r"(r[32 * h + 24]), "=r"(r[32 * h + 25]), "=r"(r[32 * h + 26]), "=r"(r[32 * h + 27]),
               "=r"(r[32 * h + 28]), "=r"(r[32 * h + 29]), "=r"(r[32 * h + 30]), "=r"(r[32 * h + 31])
-            : "r"(taddr + 32 * h));
+            : "r"(taddr + gap * h));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
     // the values exist from here on: nothing may use them before the wait
 #pragma unroll
