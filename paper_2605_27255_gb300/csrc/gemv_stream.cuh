@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
     float* xs = reinterpret_cast<float*>(smem4);  // [NB][K], split layout
     __shared__ int head_unit[kStreamWarps], tail_unit[kStreamWarps], head_fin[kStreamWarps];
     __shared__ float head_val[kStreamWarps][RU][NB], tail_val[kStreamWarps][RU][NB];
-    __shared__ float red_v[kStreamWarps][NB];
+    __shared__ float red_v[kStreamWarps][NB], rs[kStreamWarps][NB];
     __shared__ int red_r[kStreamWarps][NB];
     // EPI_RESADD: the CTA's residual values, loaded with the input after the
     // dependency wait, so that finishing a row does not wait for a load
@@ -700,9 +700,13 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
         }
         const bool ypre_on = p.epi == EPI_RESADD && u1 - u0 <= kYpreUnits;
         __syncthreads();
-        float rs[NB];
-        stage_input_async<T, NB>(p, xs, reinterpret_cast<T*>(xs + NB * K), b0, nb, rs, ypre_on ? ypre_s : nullptr, u0,
+        float rs_f[NB];
+        stage_input_async<T, NB>(p, xs, reinterpret_cast<T*>(xs + NB * K), b0, nb, rs_f, ypre_on ? ypre_s : nullptr, u0,
                                  u1 - u0);
+        if (lane == 0)  // kept in shared memory: the weight loop has no register to spare
+#pragma unroll
+            for (int bb = 0; bb < NB; ++bb) rs[warp][bb] = rs_f[bb];
+        __syncwarp();
 
         float best_v[NB];
         int best_r[NB];
@@ -747,7 +751,7 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
                         const int r = crow % RU;
 #pragma unroll
                         for (int bb = 0; bb < NB; ++bb) {
-                            const float t = warp_sum(acc[bb]) * rs[bb];
+                            const float t = warp_sum(acc[bb]) * rs[warp][bb];
                             acc[bb] = 0.f;
 #pragma unroll
                             for (int rr = 0; rr < RU; ++rr)
@@ -792,7 +796,7 @@ __global__ void __launch_bounds__(kStreamThreads) gemv_rows_kernel(GemvParams p)
             float a[RU][NB];
 #pragma unroll
             for (int bb = 0; bb < NB; ++bb) {
-                const float t = warp_sum(acc[bb]) * rs[bb];
+                const float t = warp_sum(acc[bb]) * rs[warp][bb];
 #pragma unroll
                 for (int rr = 0; rr < RU; ++rr) a[rr][bb] = part[rr][bb] + ((rr == r && cj > 0) ? t : 0.f);
             }
