@@ -208,11 +208,14 @@ __device__ __forceinline__ int tc_park_idx(int r, int c4) {
 
 // Split-K epilogue of 4 batch columns [4*c4, 4*c4+4) of tile row rr (and, for
 // SwiGLU, its up row rr+1), summed over the cluster in split order, scaled by
-// rstd[b] (a per-sequence RMSNorm factor) when rstd is given.
+// rstd[b] (a per-sequence RMSNorm factor) when rstd is given.  EPI_ARGMAX:
+// best[j] keeps the largest key of column 4 c4 + j over the thread's items (a
+// thread has the same c4 in all of them), see tc_cluster_argmax.
 template <int BH>
 __device__ __forceinline__ void tc_cluster_epilogue(const TcParams& p, cooperative_groups::cluster_group& cl,
                                                     float* park, int tile, int rr, int c4,
-                                                    const float* rstd = nullptr, const float* ypre = nullptr) {
+                                                    unsigned long long (&best)[4], const float* rstd = nullptr,
+                                                    const float* ypre = nullptr) {
     // every split's distributed-shared-memory load is issued before any is
     // used (a remote load takes several hundred cycles), then the splits are
     // added in split order (deterministic)
@@ -259,11 +262,30 @@ __device__ __forceinline__ void tc_cluster_epilogue(const TcParams& p, cooperati
             case EPI_RESADD: *yp = (ypre ? ypre[j] : *yp) + va[j]; break;
             case EPI_ARGMAX:
                 if (p.dbg) p.dbg[(size_t)b * p.ld_dbg + row] = va[j];
-                atomicMax(p.am + b, argmax_key(va[j], row));
+                best[j] = max(best[j], argmax_key(va[j], row));
                 break;
             default: break;
         }
     }
+}
+
+// Split-K LM head, after the items: the 128 epilogue threads (et = 0 .. 127) join
+// their best keys in shared memory, one global atomicMax per CTA and sequence.
+// (An atomic per row and sequence serialised at the keys: 93 us per launch at
+// V = 4096, B = 64, now 14.9.)
+template <int BH>
+__device__ __forceinline__ void tc_cluster_argmax(const TcParams& p, int et, const unsigned long long (&best)[4],
+                                                  unsigned long long* amx) {
+    for (int b = et; b < BH; b += 128) amx[b] = 0ull;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    static_assert(128 % (BH / 4) == 0, "a thread keeps its columns over its items");
+    const int c4 = et % (BH / 4);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (best[j]) atomicMax(amx + 4 * c4 + j, best[j]);
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    for (int b = et; b < BH && b < p.B; b += 128)
+        if (amx[b]) atomicMax(p.am + b, amx[b]);
 }
 
 // BH: batch columns (a multiple of 16, >= B); the MMA N is 2 * BH (hi | lo).
@@ -285,6 +307,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
     __shared__ uint32_t tmem_base;
     __shared__ float red_v[4][BH];
     __shared__ int red_r[4][BH];
+    __shared__ unsigned long long amx[BH];
     PIPO_TR(__shared__ unsigned long long tr_s[3]; const TraceT0 tr0 = trace_begin();)
 
     pdl_launch();
@@ -417,10 +440,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
         const int r0 = min(kTcM, split * R), r1 = min(kTcM, r0 + R);
         const int step = p.ru == 2 ? 2 : 1;
         const int items = (r1 - r0) / step * (BH / 4);
+        unsigned long long best[4] = {0ull, 0ull, 0ull, 0ull};
         for (int it = threadIdx.x; it < items; it += kTcThreads) {
             const int rr = r0 + (it / (BH / 4)) * step, c4 = it % (BH / 4);
-            tc_cluster_epilogue<BH>(p, cl, park, tile, rr, c4);
+            tc_cluster_epilogue<BH>(p, cl, park, tile, rr, c4, best);
         }
+        if (p.epi == EPI_ARGMAX) tc_cluster_argmax<BH>(p, (int)threadIdx.x, best, amx);
         cl.sync();  // no CTA leaves while others still read its shared memory
     }
     PIPO_TR(if (threadIdx.x == 0) tr_s[2] = trace_now();)
@@ -483,6 +508,7 @@ __global__ void __launch_bounds__(kTcfThreads, 1)
     __shared__ uint32_t tmem_base;
     __shared__ float red_v[4][BH];
     __shared__ int red_r[4][BH];
+    __shared__ unsigned long long amx[BH];
     __shared__ float ss_s[BH], rstd_s[BH];
     // EPI_RESADD: the residual values this thread's epilogue updates, loaded
     // right after the dependency wait so that the epilogue does not wait for them
@@ -750,14 +776,16 @@ __global__ void __launch_bounds__(kTcfThreads, 1)
             const int r0 = min(kTcM, split * R), r1 = min(kTcM, r0 + R);
             const int step = p.ru == 2 ? 2 : 1;
             const int items = (r1 - r0) / step * (BH / 4);
+            unsigned long long best[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
             for (int k = 0; k < kPreItems; ++k) {
                 const int it = xt + 128 * k;
                 if (it >= items) break;
                 const int rr = r0 + (it / (BH / 4)) * step, c4 = it % (BH / 4);
-                tc_cluster_epilogue<BH>(p, cl, park, tile, rr, c4, rstd_s,
+                tc_cluster_epilogue<BH>(p, cl, park, tile, rr, c4, best, rstd_s,
                                         p.epi == EPI_RESADD ? ypre + 4 * k : nullptr);
             }
+            if (p.epi == EPI_ARGMAX) tc_cluster_argmax<BH>(p, xt, best, amx);
             PIPO_TR(if (threadIdx.x == 64) tr_e[2] = trace_now();)
         }
         cl.sync();  // no CTA leaves while others still read its shared memory

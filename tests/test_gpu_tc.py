@@ -210,3 +210,21 @@ def test_decode_path_uses_tensor_core_kernels():
         assert "projections=gemv_rows_kernel" in d and "attention=attn_mma_kernel cluster=8 stages=20" in d, d
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("B,V", [(2, 24), (17, 1000), (32, 4096), (33, 129), (64, 4097)])
+def test_lm_head_tokens_are_the_argmax_of_the_logits(B, V):
+    """Vocabularies small enough for K splits, with ragged last tiles: every
+    argmax is the first largest of the GPU's own logits (exact)."""
+    s = MID.with_(V=V)
+    w = synth.gen_weights(s, seed=5)
+    gpu = capi.Pipo(s, w, max_batch=B, max_ctx=8, debug=True)
+    try:
+        gpu.prefill(synth.gen_prompts(B, 4, s.V, seed=6).numpy())
+        for _ in range(2):
+            gpu.step()
+            d = gpu.debug()
+            for lg, x in (("logits_b", "x_b"), ("logits_d", "x_d")):
+                assert (d[lg].argmax(1) == d[x]).all(), x
+    finally:
+        gpu.close()
