@@ -73,7 +73,7 @@ def parse():
                     help="timed replays of the projection-only graph for the roofline (default: the step count, "
                          "at most 256)")
     ap.add_argument("--prefill-rows", type=int, default=128,
-                    help="prefill in chunks of this many rows (positions x sequences, at most 128); "
+                    help="prefill in chunks of this many rows (positions x sequences, at most 2048); "
                          "0: one position at a time")
     ap.add_argument("--sampler", action="store_true",
                     help="decode with the paper's evaluation sampler in both heads (T 1, top-k 20, top-p 0.95, "
