@@ -246,18 +246,47 @@ __global__ void __launch_bounds__(kBlkThreads, 1) gemv_kernel(GemvParams p, int 
                         rstd_s[qb][g] = 1.0f / sqrtf((ss_s[2 * qb][g] + ss_s[2 * qb + 1][g]) / (float)len + p.eps);
                     }
                     __syncthreads();
-                    for (int q = half * 32 + lane; q < kpad / 4; q += 64) {
-                        const int k = k0 + 4 * q;
-                        if (k >= K) break;
-                        const int g = (p.joint_norm || k < K0) ? 0 : 1;
-                        if (!(g == 0 ? norm0 : norm1)) continue;
-                        const size_t kk = (size_t)(p.joint_norm || g == 0 ? k : k - K0);
-                        const float4 gm = wide ? ld4<T>(p.seg[g].gamma, kk) : ld4_scalar<T>(p.seg[g].gamma, kk);
-                        float4* xp = xat(q);
-                        const float r = rstd_s[bb][g];
-                        float4 v = *xp;
-                        v.x *= r * gm.x; v.y *= r * gm.y; v.z *= r * gm.z; v.w *= r * gm.w;
-                        *xp = v;
+                    if constexpr (sizeof(T) == 4) {
+                        // four gain loads in flight: six sequences, four layers of H = 1024,
+                        // 248 -> 242 us per step; eight bf16 rows (4B widths) 0.4 % slower with it
+                        for (int q = half * 32 + lane; q < kpad / 4; q += 64 * 4) {
+                            float4 gm[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int k = k0 + 4 * (q + 64 * u);
+                                const int g = (p.joint_norm || k < K0) ? 0 : 1;
+                                gm[u] = make_float4(1.f, 1.f, 1.f, 1.f);
+                                if (q + 64 * u < kpad / 4 && k < K && (g == 0 ? norm0 : norm1)) {
+                                    const size_t kk = (size_t)(p.joint_norm || g == 0 ? k : k - K0);
+                                    gm[u] = wide ? ld4<T>(p.seg[g].gamma, kk) : ld4_scalar<T>(p.seg[g].gamma, kk);
+                                }
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int qq = q + 64 * u, k = k0 + 4 * qq;
+                                const int g = (p.joint_norm || k < K0) ? 0 : 1;
+                                if (qq >= kpad / 4 || k >= K || !(g == 0 ? norm0 : norm1)) continue;
+                                float4* xp = xat(qq);
+                                const float r = rstd_s[bb][g];
+                                float4 v = *xp;
+                                v.x *= r * gm[u].x; v.y *= r * gm[u].y; v.z *= r * gm[u].z; v.w *= r * gm[u].w;
+                                *xp = v;
+                            }
+                        }
+                    } else {
+                        for (int q = half * 32 + lane; q < kpad / 4; q += 64) {
+                            const int k = k0 + 4 * q;
+                            if (k >= K) break;
+                            const int g = (p.joint_norm || k < K0) ? 0 : 1;
+                            if (!(g == 0 ? norm0 : norm1)) continue;
+                            const size_t kk = (size_t)(p.joint_norm || g == 0 ? k : k - K0);
+                            const float4 gm = wide ? ld4<T>(p.seg[g].gamma, kk) : ld4_scalar<T>(p.seg[g].gamma, kk);
+                            float4* xp = xat(q);
+                            const float r = rstd_s[bb][g];
+                            float4 v = *xp;
+                            v.x *= r * gm.x; v.y *= r * gm.y; v.z *= r * gm.z; v.w *= r * gm.w;
+                            *xp = v;
+                        }
                     }
                 }
             }
