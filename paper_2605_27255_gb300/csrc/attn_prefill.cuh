@@ -33,6 +33,7 @@
 #pragma once
 
 #include "attn_mma.cuh"
+#include "copy_ring.cuh"
 #include "tcgen05_gemm.cuh"
 
 namespace pipo {
@@ -189,26 +190,21 @@ __global__ void __launch_bounds__(kPfThreads, 1) attn_prefill_kernel(AttnParams 
                     tma_load_2d(dst + kPfHalf + i * kMmaHalf, tm, 64, trow, bar);
                 }
             };
-            int t = 0;
-            for (; t < nt; ++t) {
-                const int st = t % kPfStages;
-                const uint32_t ph = (uint32_t)(((t / kPfStages) & 1) ^ 1);
-                if (t >= kPfStages && !mbar_wait(k_empty + st, ph, 41, t)) break;
-                load(&tmK, k_s + st * kPfTile, k_full + st, t);
-                if (t >= kPfStages && !mbar_wait(v_empty + st, ph, 41, t)) break;
-                load(&tmV, v_s + st * kPfTile, v_full + st, t);
-            }
-            // no copy into this CTA's shared memory may still be in flight at exit
-            for (int i = max(0, nt - kPfStages); i < t; ++i) {
-                mbar_wait(k_full + i % kPfStages, (uint32_t)((i / kPfStages) & 1), 42, i);
-                mbar_wait(v_full + i % kPfStages, (uint32_t)((i / kPfStages) & 1), 42, i);
-            }
+            // (no copy into this CTA's shared memory is in flight at its end)
+            ring_fill_pair<kPfStages>(
+                nt, [&](int v, int st, uint32_t ph, int t) { return mbar_wait((v ? v_empty : k_empty) + st, ph, 41, t); },
+                [&](int v, int st, int t) {
+                    if (v) load(&tmV, v_s + st * kPfTile, v_full + st, t);
+                    else load(&tmK, k_s + st * kPfTile, k_full + st, t);
+                },
+                [&](int v, int st, uint32_t ph, int t) { mbar_wait((v ? v_full : k_full) + st, ph, 42, t); });
         } else if (warp == 1 && lane == 0) {
             // ---- MMA issuer.  TMEM: scores / probabilities of tile t at
             // (t & 1) * 128, its T tile at 256 + (t & 1) * 128
             constexpr uint32_t id_s = umma_idesc_bf16(kPfVec, kPfEnt);
             constexpr uint32_t id_o = umma_idesc_bf16(kPfVec, DH) | (1u << 16);  // B MN-major
             const uint32_t q0 = smem_u32(q_s), k0 = smem_u32(k_s), v0 = smem_u32(v_s);
+            int ns = 0, no = 0;  // score and output tiles committed
             auto scores = [&](int t) {
                 const int st = t % kPfStages;
                 if (!mbar_wait(k_full + st, (uint32_t)((t / kPfStages) & 1), 43, t)) return false;
@@ -224,6 +220,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) attn_prefill_kernel(AttnParams 
                     }
                 umma_commit(s_full + (t & 1));
                 umma_commit(k_empty + st);
+                ns = t + 1;
                 return true;
             };
             bool ok = scores(0);
@@ -244,13 +241,13 @@ __global__ void __launch_bounds__(kPfThreads, 1) attn_prefill_kernel(AttnParams 
                                      (part > 0 || k > 0) ? 1u : 0u);
                 umma_commit(o_full + (t & 1));
                 umma_commit(v_empty + st);
+                no = t + 1;
                 if (t + 2 < nt)  // the scores over this tile's probabilities, once they are read
                     ok = mbar_wait(o_full + (t & 1), (uint32_t)((t >> 1) & 1), 45, t) && scores(t + 2);
             }
             // every commit into this CTA's barriers has arrived before the end
-            for (int i = max(0, nt - kPfStages); i < nt && ok; ++i)
-                ok = mbar_wait(k_empty + i % kPfStages, (uint32_t)((i / kPfStages) & 1), 45, i) &&
-                     mbar_wait(v_empty + i % kPfStages, (uint32_t)((i / kPfStages) & 1), 45, i);
+            ring_drain<kPfStages>(ns, [&](int st, uint32_t ph, int t) { mbar_wait(k_empty + st, ph, 45, t); });
+            ring_drain<kPfStages>(no, [&](int st, uint32_t ph, int t) { mbar_wait(v_empty + st, ph, 45, t); });
         }
         __syncwarp();
     } else {
