@@ -46,4 +46,15 @@ PIPO_RING_FN void ring_fill_pair(int nt, Empty empty, Load load, Full full) {
     ring_drain<ST>(n1, [&](int st, uint32_t ph, int t) { full(1, st, ph, t); });
 }
 
+// The end of a CTA pair's copying threads after n stages each: the leader waits
+// for every copy (both CTAs' arrive on its barriers), whatever gave up before;
+// then each CTA for the commits that freed its stages, which come in order, so
+// that after one that never came there are none.
+template <int ST, class Full, class Empty>
+PIPO_RING_FN void pair_drain(int n, bool leader, Full full, Empty empty) {
+    if (leader) ring_drain<ST>(n, full);
+    bool ok = true;
+    ring_drain<ST>(n, [&](int st, uint32_t ph, int i) { ok = ok && empty(st, ph, i); });
+}
+
 }  // namespace pipo

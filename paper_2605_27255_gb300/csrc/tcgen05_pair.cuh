@@ -34,6 +34,7 @@
 // any width (the weight operand bounds them).
 #pragma once
 
+#include "copy_ring.cuh"
 #include "tcgen05_gemm.cuh"
 
 namespace pipo {
@@ -228,12 +229,12 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                         load_x(s, i, n);
                     }
                 }
-                // no copy into the pair's shared memory and no commit to its
+                // no copy into the pair's shared memory (they arrive on the leader's
+                // barriers, the other CTA leaves after it) and no commit to its
                 // barriers may still be in flight at exit
-                for (int i = max(0, it - ST); i < it; ++i) {
-                    if (half == 0 && !mbar_wait(full + (i % ST), (uint32_t)((i / ST) & 1), 32, i)) break;
-                    if (!mbar_wait(empty + (i % ST), (uint32_t)((i / ST) & 1), 36, i)) break;
-                }
+                pair_drain<ST>(
+                    it, half == 0, [&](int st, uint32_t ph, int i) { mbar_wait(full + st, ph, 32, i); },
+                    [&](int st, uint32_t ph, int i) { return mbar_wait(empty + st, ph, 36, i); });
             }
             __syncwarp();
         } else if (warp == 1) {
@@ -531,10 +532,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                     load_x(s, kb0 + i);
                 }
             }
-            for (int i = max(0, it - ST); i < it; ++i) {
-                if (half == 0 && !mbar_wait(full + (i % ST), (uint32_t)((i / ST) & 1), 32, i)) break;
-                if (!mbar_wait(empty + (i % ST), (uint32_t)((i / ST) & 1), 36, i)) break;
-            }
+            pair_drain<ST>(
+                it, half == 0, [&](int st, uint32_t ph, int i) { mbar_wait(full + st, ph, 32, i); },
+                [&](int st, uint32_t ph, int i) { return mbar_wait(empty + st, ph, 36, i); });
         }
         __syncwarp();
     } else if (warp == 1) {

@@ -1,6 +1,7 @@
-"""The end of the prefill attention's copy rings (csrc/copy_ring.cuh, the code
-the kernel runs), compiled for the host with waits that give up at every
-point: no copy may be in flight when the filling thread is done."""
+"""The end of the copy rings of the prefill attention and of the CTA-pair GEMMs
+(csrc/copy_ring.cuh, the code the kernels run), compiled for the host with
+waits that give up at every point: no copy may be in flight when the filling
+thread is done."""
 import os
 import subprocess
 
@@ -39,8 +40,39 @@ static int run(int nt, int fail, bool lost) {
         for (int x : c) bad += x != 2;
     return bad;
 }
+// a pair's leader after n stages, the commits from stage `gone` on never made: copies not waited for,
+// waits for commits after one that gave up
+template <int S>
+static int pair(int n, int gone, bool leader) {
+    std::vector<int> state(n, 1);
+    int bad = 0, last = -1;
+    bool over = false;
+    pipo::pair_drain<S>(
+        n, leader,
+        [&](int st, uint32_t ph, int i) {
+            if (i < 0 || i >= n || st != i % S || ph != (uint32_t)((i / S) & 1)) ++bad;
+            else state[i] = 2;
+            return false;  // a full barrier that gives up does not end the waiting
+        },
+        [&](int st, uint32_t ph, int i) {
+            if (over || i < n - S || i <= last || st != i % S || ph != (uint32_t)((i / S) & 1)) ++bad;
+            last = i;
+            over = i >= gone;
+            return !over;
+        });
+    for (int i = n > S ? n - S : 0; i < n; ++i) bad += leader && state[i] != 2;
+    if (n > 0 && gone >= n) bad += last != n - 1;
+    return bad;
+}
 int main() {
     int bad = 0, runs = 0;
+    for (int n = 0; n <= 20; ++n)
+        for (int gone = 0; gone <= n; ++gone)
+            for (int leader = 0; leader < 2; ++leader) {
+                const int b = pair<4>(n, gone, leader) + pair<6>(n, gone, leader) + pair<8>(n, gone, leader);
+                if (b) std::printf("pair n=%d gone=%d leader=%d: %d\n", n, gone, leader, b);
+                bad += b;
+            }
     for (int nt = 0; nt <= 9; ++nt)
         for (int fail = -1; fail < 2 * nt; ++fail)
             for (int lost = 0; lost < 2; ++lost) {
