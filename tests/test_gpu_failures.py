@@ -4,6 +4,7 @@ the device (nothing here faults, traps or hangs a GPU):
 * a bounded device wait given a short limit on an mbarrier that nothing
   completes gives up, records its site and is reported as PIPO_ECUDA; the
   same wait on a completed barrier reports nothing; the device stays usable;
+  a step that finds such an error reports it, once;
 * an out-of-memory on the k-th device allocation of pipo_init (injected on
   the host, PIPO_TEST_FAIL_ALLOC) returns PIPO_ENOMEM, frees everything
   allocated before it (device memory back to where it was, repeatedly), and
@@ -58,6 +59,29 @@ def test_bounded_wait_gives_up_and_reports_its_site():
     assert capi.pipo_selftest_wait(0, 0)[0] == capi.PIPO_EINVAL
     # the context survives: a decode runs and matches the oracle
     _tiny_step_matches_oracle()
+
+
+@pytest.mark.parametrize("taken_by", ["counters", "step"])
+def test_a_wait_that_gave_up_is_reported_once(monkeypatch, taken_by):
+    """The error of an asynchronous step is reported by the next call that
+    asks, the counters or a synchronous step, with the wait's site, and by no
+    call after it."""
+    s = synth.TINY
+    g = capi.Pipo(s, synth.gen_weights(s, seed=0), max_batch=1, max_ctx=16)
+    try:
+        g.prefill(synth.gen_prompts(1, 8, s.V, seed=1).numpy())
+        monkeypatch.setenv("PIPO_TEST_KEEP_WAIT_ERROR", "1")
+        assert capi.pipo_selftest_wait(0, 1_000_000)[0] == capi.PIPO_OK  # gave up; left for the step to find
+        monkeypatch.delenv("PIPO_TEST_KEEP_WAIT_ERROR")
+        g.step_async()
+        with pytest.raises(capi.PipoError) as e:
+            g.counters() if taken_by == "counters" else g.step()
+        assert e.value.status == capi.PIPO_ECUDA and "wait site 90" in str(e.value)
+        g.step()
+        g.counters()
+        g.step()
+    finally:
+        g.close()
 
 
 def test_injected_allocation_failure_frees_everything(monkeypatch):
