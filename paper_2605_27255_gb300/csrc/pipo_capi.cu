@@ -315,6 +315,7 @@ constexpr size_t kXsBudget = 100 * 1024;      // fp32 bytes of the longest GEMV 
 // shared memory of the staged register-ring attention (the CTA's slice of
 // cached keys and values); longer slices take the register ring alone
 constexpr size_t kAttnStageMax = 160 * 1024;
+constexpr int kTcMaxBatch = 128;              // sequences whose steps run on the tensor-core projections
 constexpr int kMaxPrefillRows = 2048;         // rows of a prefill chunk (PIPO_PREFILL_ROWS)
 constexpr int kAutoRows = 512;                // ... that the library chooses by itself
 constexpr size_t kBlkSmemMax = (size_t)kBlkKMax * kBlkNB * 4 + (size_t)kBlkSeg * 32 * 4;
@@ -845,7 +846,7 @@ bool tc_eligible(const pipo_ctx* ctx, const GemvParams& p) {
     if (ctx->rows_fp32) return false;
     // decode batches above 128 keep the fp32 products of the CUDA-core GEMV;
     // prefill chunks may be as tall as their buffers
-    const int most = ctx->rows > ctx->B ? ctx->tc_bn_max : std::min(ctx->tc_bn_max, 128);
+    const int most = ctx->rows > ctx->B ? ctx->tc_bn_max : std::min(ctx->tc_bn_max, kTcMaxBatch);
     return ctx->cfg.dtype == 1 && ctx->tc_xb && p.B >= ctx->tc_min_b && p.B <= most &&
            p.K % kTcBK == 0 && p.K <= ctx->tc_kmax && p.K <= 4 * kPrepQ * kPrepThreads && rows >= kTcM;
 }
@@ -1736,9 +1737,16 @@ pipo_status enqueue_prefill_chunk(pipo_ctx* ctx, bool regular, int j0, int C) {
 // cores takes chunks of up to kAutoRows on them, and one whose steps keep
 // fp32 products (a single sequence, fp32 models) one weight pass of the
 // row-block GEMV, eight rows.
+//
+// A batch of more than 128 has fp32 products in its steps too, and more
+// sequences than a weight pass: no chunks (0), position by position.  Chunks of
+// hi and lo products were 6 to 10 times as fast there and three times as far from 64
+// bits (two 4B-wide layers, 160 sequences of 20 tokens: 73 ms and 1.4e-4
+// against 11 ms and 4.3e-4).
 constexpr int kChunkK = 4300;
 int prefill_chunk_rows(const pipo_ctx* ctx) {
     const pipo_config& c = ctx->cfg;
+    if (c.dtype == 1 && ctx->B > kTcMaxBatch) return 0;
     if (ctx->prefill_auto && (c.dtype != 1 || ctx->B < ctx->tc_min_b)) return kBlkNB;
     if (ctx->prefill_rows < 2 * kPairN || c.dtype != 1) return ctx->prefill_rows;
     const int pairs = std::max(1, pair_max_clusters()), qd = c.n_q_heads * c.head_dim, kd = c.n_kv_heads * c.head_dim;

@@ -49,10 +49,10 @@ def test_chunked_pair_prefill_tiny_fp32(monkeypatch, variant):
 
 
 def _prefill_state(shape, w, prompts, rows, regular=False):
-    if rows:
+    """rows: PIPO_PREFILL_ROWS (0: one position at a time), None: not set."""
+    os.environ.pop("PIPO_PREFILL_ROWS", None)
+    if rows is not None:
         os.environ["PIPO_PREFILL_ROWS"] = str(rows)
-    else:
-        os.environ.pop("PIPO_PREFILL_ROWS", None)
     B, T = prompts.shape
     n = T if regular else (T + 1) // 2
     g = capi.Pipo(shape, w, max_batch=B, max_ctx=n + 4, debug=True)
@@ -104,6 +104,23 @@ def test_chunked_equals_position_by_position(regular):
             assert np.abs(Va - Vb).max() <= 2 * tol * scale
     assert np.abs(a[1]["logits_b"] - b[1]["logits_b"]).max() <= 2 * tol
     assert list(a[4][0]) == list(b[4][0])  # cache lengths
+
+
+@pytest.mark.parametrize("rows", [None, 2048])
+def test_batches_above_128_keep_the_products_of_their_steps(rows):
+    """More than 128 sequences: the prompt goes position by position with the
+    fp32 products of the batch's steps, whatever the chunk setting (bit for
+    bit)."""
+    s = MID
+    w = synth.gen_weights(s, seed=5)
+    prompts = synth.gen_prompts(130, 9, s.V, seed=9).numpy()
+    a = _prefill_state(s, w, prompts, 0)
+    b = _prefill_state(s, w, prompts, rows)
+    for key in ("logits_b", "h_b", "h_d", "conf"):
+        assert np.array_equal(a[1][key], b[1][key]), key
+    for cb_a, cb_b in zip(a[2], b[2]):
+        for (Ka, Va), (Kb, Vb) in zip(cb_a, cb_b):
+            assert np.array_equal(Ka, Kb) and np.array_equal(Va, Vb)
 
 
 @pytest.mark.parametrize("attn", ["rows", "tile"])
