@@ -438,11 +438,12 @@ PIPO_API pipo_status pipo_selftest_wait(int32_t signal, uint64_t limit_ns, uint3
 
 /* Which kernels the next decode step launches for the projections and the
  * attention, and the attention cluster size, as one NUL-terminated line of
- * at most cap bytes in h_buf, e.g. "B=16 projections=gemm_tc_kernel<16>+
- * prep_bf16_kernel (tcgen05) attention=attn_mma_kernel cluster=2
- * mode=pair heads=argmax", followed by the prefill arrangement when chunks
- * are enabled.  Batch B
- * is the prefilled batch (before a prefill: cfg.max_batch).  A report of
+ * at most cap bytes in h_buf, e.g. "B=16 projections=gemm_tcf_kernel<16>
+ * (tcgen05) attention=attn_mma_kernel cluster=2 mode=pair heads=argmax
+ * prefill=chunks of 512 rows (attn_prefill_kernel)": the prefill of a prompt
+ * of batch B, as the rows (positions x sequences) and the attention of a whole
+ * chunk ("per-row attention": that of the steps), or "one position at a
+ * time".  Batch B is the prefilled batch (before a prefill: cfg.max_batch).  A report of
  * this library's kernel choices; the paper has no counterpart.  EINVAL for
  * a NULL context or buffer or cap == 0. */
 PIPO_API pipo_status pipo_describe_step(const pipo_ctx *ctx, char *h_buf, size_t cap);

@@ -1252,10 +1252,10 @@ size_t attn_stage(const pipo_ctx* ctx, int splits, bool chunk, int* stage_max) {
 // rows 59.6 / 63.2, 64 rows 45.2 / 36.7, 128 rows 37.1 / 23.0; 4 x 2000 tokens
 // 32 rows 45.0 / 48.3, 64 rows 30.8 / 29.8; 16 x 400 tokens 64 rows (4 positions)
 // 21.7 / 22.5, 128 rows 15.3 / 15.0.
-bool prefill_tiles(const pipo_ctx* ctx, int R) {
+bool prefill_tiles(const pipo_ctx* ctx, int R, int B) {
     if (!attn_mma_ok(ctx) || (int)ctx->kv_tm.size() != 2 * ctx->n_cache_layers) return false;
     if (ctx->prefill_attn > 0) return ctx->prefill_attn == 2;
-    return R >= 64 && R / ctx->B >= 8;
+    return R >= 64 && R / B >= 8;
 }
 
 // Rows the bf16 hi part of a projection's prepared operand takes before its lo
@@ -1320,7 +1320,7 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
             bool was;
             ~PdlGuard() { c->pdl = was; }
         } guard{ctx, ctx->pdl};
-        if (ctx->pdl_eager && !(chunk && prefill_tiles(ctx, R))) ctx->pdl = false;
+        if (ctx->pdl_eager && !(chunk && prefill_tiles(ctx, R, ctx->B))) ctx->pdl = false;
         ctx->prof_kind = 1;
         ctx->prof_bytes = 0.0;
         for (int b = 0; b < ctx->B && b < (int)ctx->h_len.size(); ++b)
@@ -1337,14 +1337,14 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
         ap.no_append = chunk ? 1 : 0;
         void* args[] = {&ap};
         const int cs = attn_cluster_size(ctx, R);
-        const bool mma = (chunk && prefill_tiles(ctx, R)) ||
+        const bool mma = (chunk && prefill_tiles(ctx, R, ctx->B)) ||
                          (attn_use_mma(ctx, R) &&
                           (cs <= 8 || (!chunk && (attn_balanced_slots(ctx, R) > 0 || attn_mma_flat_splits(ctx, R) > 0))));
         if (!mma) o_hi = 0;  // the other attention kernels write fp32
         // a tile attention that leaves SMs idle keeps the preparation: without
         // it the O projection's CTAs settle, two to an SM, on the SMs that the
         // attention does not use (4 x 1024 tokens, 32 CTAs: 14.48 against 14.84 ms)
-        if (chunk && prefill_tiles(ctx, R)) {
+        if (chunk && prefill_tiles(ctx, R, ctx->B)) {
             const int TP = kPfVec / (c.n_q_heads / c.n_kv_heads), C = R / ctx->B;
             if ((long long)((C + TP - 1) / TP) * c.n_kv_heads * ctx->B < ctx->sms) o_hi = 0;
         }
@@ -1353,7 +1353,7 @@ pipo_status enqueue_block(pipo_ctx* ctx, const BlockW& bw, int cache_layer, floa
             ap.out_lo = (size_t)o_hi * qd;
         }
         const int G = c.n_q_heads / c.n_kv_heads;
-        if (chunk && prefill_tiles(ctx, R)) {
+        if (chunk && prefill_tiles(ctx, R, ctx->B)) {
             // causal tiles: the positions of a tile share every key and value they read
             void* fn = k_pick_attn_prefill(G);
             CK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prefill_attn_smem()));
@@ -1744,10 +1744,10 @@ pipo_status enqueue_prefill_chunk(pipo_ctx* ctx, bool regular, int j0, int C) {
 // bits (two 4B-wide layers, 160 sequences of 20 tokens: 73 ms and 1.4e-4
 // against 11 ms and 4.3e-4).
 constexpr int kChunkK = 4300;
-int prefill_chunk_rows(const pipo_ctx* ctx) {
+int prefill_chunk_rows(const pipo_ctx* ctx, int B) {
     const pipo_config& c = ctx->cfg;
-    if (c.dtype == 1 && ctx->B > kTcMaxBatch) return 0;
-    if (ctx->prefill_auto && (c.dtype != 1 || ctx->B < ctx->tc_min_b)) return kBlkNB;
+    if (c.dtype == 1 && B > kTcMaxBatch) return 0;
+    if (ctx->prefill_auto && (c.dtype != 1 || B < ctx->tc_min_b)) return kBlkNB;
     if (ctx->prefill_rows < 2 * kPairN || c.dtype != 1) return ctx->prefill_rows;
     const int pairs = std::max(1, pair_max_clusters()), qd = c.n_q_heads * c.head_dim, kd = c.n_kv_heads * c.head_dim;
     const int shp[4][2] = {{qd + 2 * kd, c.hidden}, {c.hidden, qd}, {2 * c.ffn, c.hidden}, {c.hidden, c.ffn}};
@@ -1767,14 +1767,20 @@ int prefill_chunk_rows(const pipo_ctx* ctx) {
     return best;
 }
 
-// The positions before a prompt's last one in chunks of prefill_rows / B
-// positions (when chunks are enabled and hold two or more positions);
-// *j receives the first position left for the position-by-position path.
+// Positions of a whole chunk for a batch of B; 0: one position at a time.
+int prefill_chunk_positions(const pipo_ctx* ctx, int B) {
+    const int C = prefill_chunk_rows(ctx, B) / B;
+    return C < 2 || ctx->attn_v0 ? 0 : C;
+}
+
+// The positions before a prompt's last one in chunks (where chunks hold two or
+// more positions); *j receives the first position left for the
+// position-by-position path.
 pipo_status enqueue_prefill_chunks(pipo_ctx* ctx, bool regular, int N, int* j) {
     const int B = ctx->B;
-    const int cmax = prefill_chunk_rows(ctx) / B;
+    const int cmax = prefill_chunk_positions(ctx, B);
     *j = 0;
-    if (cmax < 2 || ctx->attn_v0) return PIPO_OK;
+    if (cmax == 0) return PIPO_OK;
     while (N - 1 - *j >= 2) {
         const int C = std::min(cmax, N - 1 - *j);
         TRY(enqueue_prefill_chunk(ctx, regular, *j, C));
@@ -3017,9 +3023,11 @@ pipo_status pipo_describe_step(const pipo_ctx* ctx, char* h_buf, size_t cap) {
     // decoding mode, heads and prefill arrangement
     d += ctx->regular ? " mode=regular" : " mode=pair";
     d += ctx->samp_on ? " heads=sampled" : " heads=argmax";
-    if (ctx->prefill_rows >= 2 && !ctx->prefill_auto)
-        d += " prefill=chunks of " + std::to_string(ctx->prefill_rows) + " rows (" +
-             (ctx->prefill_attn != 1 && attn_mma_ok(ctx) ? "attn_prefill_kernel" : "per-row attention") + ")";
+    const int chunk = prefill_chunk_positions(ctx, B);
+    if (chunk == 0) d += " prefill=one position at a time";
+    else
+        d += " prefill=chunks of " + std::to_string(chunk * B) + " rows (" +
+             (prefill_tiles(ctx, chunk * B, B) ? "attn_prefill_kernel" : "per-row attention") + ")";
     snprintf(h_buf, cap, "%s", d.c_str());
     return PIPO_OK;
 }

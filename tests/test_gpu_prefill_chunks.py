@@ -7,6 +7,7 @@ steps that read the chunk-written caches), against the position-by-position
 prefill of the same context shape (cache contents and outputs), for pair and
 regular decoding, with ragged last chunks and several sequences.
 """
+import functools
 import os
 
 import numpy as np
@@ -104,6 +105,36 @@ def test_chunked_equals_position_by_position(regular):
             assert np.abs(Va - Vb).max() <= 2 * tol * scale
     assert np.abs(a[1]["logits_b"] - b[1]["logits_b"]).max() <= 2 * tol
     assert list(a[4][0]) == list(b[4][0])  # cache lengths
+
+
+ONE = "prefill=one position at a time"
+TILES, ROWS = "prefill=chunks of %d rows (attn_prefill_kernel)", "prefill=chunks of %d rows (per-row attention)"
+
+
+@pytest.mark.parametrize("rows,attn,B,want", [
+    (None, None, 1, ROWS % 8), (None, None, 2, TILES % 512), (None, None, 3, TILES % 510), (None, None, 128, ROWS % 512),
+    (None, None, 130, ONE), (0, None, 2, ONE), (2, None, 2, ONE), (24, None, 3, ROWS % 24), (24, "tile", 3, TILES % 24),
+    (63, None, 1, ROWS % 63), (64, None, 1, TILES % 64), (128, None, 32, ROWS % 128), (300, None, 1, TILES % 300),
+    (300, "rows", 1, ROWS % 300), (128, None, 130, ONE)])
+def test_describe_names_the_prefill_that_runs(monkeypatch, rows, attn, B, want):
+    """The chunk the library takes (not the one asked for) and its attention,
+    at the borders of both rules."""
+    monkeypatch.delenv("PIPO_PREFILL_ROWS", raising=False)
+    monkeypatch.delenv("PIPO_PREFILL_ATTN", raising=False)
+    if rows is not None:
+        monkeypatch.setenv("PIPO_PREFILL_ROWS", str(rows))
+    if attn:
+        monkeypatch.setenv("PIPO_PREFILL_ATTN", attn)
+    g = capi.Pipo(MID, _weights_once(), max_batch=B, max_ctx=40)
+    try:
+        assert g.describe().endswith(want), g.describe()
+    finally:
+        g.close()
+
+
+@functools.lru_cache(maxsize=1)
+def _weights_once():
+    return synth.gen_weights(MID, seed=5)
 
 
 @pytest.mark.parametrize("rows", [None, 2048])
