@@ -58,6 +58,14 @@ NOMINAL_HBM_GBS = 8000.0  # GB300 HBM3e nominal (~8 TB/s), context beside the me
 REF_BUDGET_S = 150.0      # reference arm: about this many seconds of timed oracle steps
 
 
+def set_prefill_rows(rows: int) -> None:
+    """PIPO_PREFILL_ROWS for --prefill-rows (0 is a setting, -1 is none)."""
+    if rows < 0:
+        os.environ.pop("PIPO_PREFILL_ROWS", None)
+    else:
+        os.environ["PIPO_PREFILL_ROWS"] = str(rows)
+
+
 def parse():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -74,7 +82,7 @@ def parse():
                          "at most 256)")
     ap.add_argument("--prefill-rows", type=int, default=128,
                     help="prefill in chunks of this many rows (positions x sequences, at most 2048); "
-                         "0: one position at a time")
+                         "0: one position at a time; -1: the library's own choice (named in roofline.kernel)")
     ap.add_argument("--sampler", action="store_true",
                     help="decode with the paper's evaluation sampler in both heads (T 1, top-k 20, top-p 0.95, "
                          "repetition penalty 1.5; seeded draws) instead of the greedy argmax")
@@ -404,8 +412,7 @@ def run_pipo(args):
         max_ctx = max(max_ctx, T + W + K + 8)  # regular decoding: one cache entry per token
 
     w = build_weights(shape, "cuda")
-    if args.prefill_rows:
-        os.environ["PIPO_PREFILL_ROWS"] = str(args.prefill_rows)  # read when the context is created
+    set_prefill_rows(args.prefill_rows)  # read when the context is created
     g = capi.Pipo(shape, w, max_batch=B, max_ctx=max_ctx, tau=tau, force_mode=args.force)
     w_host = None
     if rank == 0 and not args.no_cpu_baseline:

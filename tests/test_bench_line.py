@@ -117,3 +117,13 @@ def test_reference_arm_runs_on_cpu_and_prints_one_contract_line():
     assert line["cpu_baseline"]["kind"] == "oracle" and line["cpu_baseline"]["value"] == line["value"]
     assert line["e2e"] == {"value": line["value"], "unit": line["unit"], "h2d_bytes_per_step": 0,
                            "d2h_bytes_per_step": 0}
+
+
+@pytest.mark.parametrize("rows,env", [(0, "0"), (128, "128"), (-1, None)])
+def test_prefill_rows_zero_is_one_position_at_a_time(monkeypatch, rows, env):
+    """--prefill-rows 0 reaches the library as 0: unset means chunks of its choice."""
+    import os
+
+    monkeypatch.setenv("PIPO_PREFILL_ROWS", "64")
+    bench.set_prefill_rows(rows)
+    assert os.environ.get("PIPO_PREFILL_ROWS") == env
