@@ -74,8 +74,9 @@ def compare(shape, tau, o, d, tok, nacc, force, stats, tol, where=""):
 
 
 def run_forced_replay(shape, weights, prompts, steps, *, tau=None, force=0, max_ctx=None,
-                      page_shuffle_seed=0, lens=None, oracle_weights=None):
-    """Prefill + `steps` decode steps on both sides; returns Stats."""
+                      page_shuffle_seed=0, lens=None, oracle_weights=None, expect=None):
+    """Prefill + `steps` decode steps on both sides; returns Stats.  expect:
+    what the context's description has to contain (the kernels meant)."""
     tau = shape.tau if tau is None else tau
     B, T = prompts.shape
     n_pairs = (T + 1) // 2
@@ -87,6 +88,7 @@ def run_forced_replay(shape, weights, prompts, steps, *, tau=None, force=0, max_
         orc = O.State(O.Model(shape, oracle_weights or weights, max_ctx=max_ctx), B)
         st = Stats()
         tok, nacc = gpu.prefill(prompts, lens)
+        assert expect is None or expect in gpu.describe(), gpu.describe()
         o = orc.prefill(prompts, lens, tau=tau, force=force)
         compare(shape, tau, o, gpu.debug(), tok, nacc, force, st, tol, "prefill")
         for i in range(steps):

@@ -23,6 +23,10 @@ MID = synth.ModelShape("mid", H=512, L=3, n_q=8, n_kv=2, d_h=128, F=1376, V=5003
                        compressor="mlp", mtp_block=1, dtype="bf16", rope_theta=1e6, tau=0.5)
 
 
+ONE = "prefill=one position at a time"
+KERNEL = {"rows": "per-row attention", "tile": "attn_prefill_kernel"}
+
+
 @pytest.mark.parametrize("attn", ["rows", "tile"])
 @pytest.mark.parametrize("rows,B,T", [(16, 1, 150), (16, 2, 149), (128, 1, 300), (128, 4, 97), (128, 16, 40)])
 def test_chunked_pair_prefill_matches_oracle(monkeypatch, attn, rows, B, T):
@@ -31,11 +35,26 @@ def test_chunked_pair_prefill_matches_oracle(monkeypatch, attn, rows, B, T):
     decode-style CTA per row, or causal tiles of positions
     (PIPO_PREFILL_ATTN=tile, attn_prefill_kernel)."""
     monkeypatch.setenv("PIPO_PREFILL_ROWS", str(rows))
-    if attn == "tile":
-        monkeypatch.setenv("PIPO_PREFILL_ATTN", "tile")
+    monkeypatch.setenv("PIPO_PREFILL_ATTN", attn)
     w = synth.gen_weights(MID, seed=3)
     prompts = synth.gen_prompts(B, T, MID.V, seed=7).numpy()
-    st = run_forced_replay(MID, w, prompts, 6)
+    st = run_forced_replay(MID, w, prompts, 6, expect=KERNEL[attn])
+    assert st.tok_checked >= 0.5 * st.tok_total
+
+
+@pytest.mark.parametrize("rows,B,T,expect", [(0, 1, 41, ONE), (0, 2, 42, ONE), (0, 5, 21, ONE),
+                                             (None, 1, 41, "prefill=chunks of 8 rows"),
+                                             (None, 2, 160, KERNEL["tile"]), (None, 70, 30, KERNEL["rows"])])
+def test_unchunked_and_default_prefill_match_oracle(monkeypatch, rows, B, T, expect):
+    """One position at a time (PIPO_PREFILL_ROWS=0: dependent launches outside
+    a graph, position after position), and what the library does by itself."""
+    monkeypatch.delenv("PIPO_PREFILL_ATTN", raising=False)
+    monkeypatch.delenv("PIPO_PREFILL_ROWS", raising=False)
+    if rows is not None:
+        monkeypatch.setenv("PIPO_PREFILL_ROWS", str(rows))
+    w = synth.gen_weights(MID, seed=3)
+    prompts = synth.gen_prompts(B, T, MID.V, seed=7).numpy()
+    st = run_forced_replay(MID, w, prompts, 2, expect=expect)
     assert st.tok_checked >= 0.5 * st.tok_total
 
 
@@ -75,6 +94,7 @@ def test_tile_attention_equals_row_attention(monkeypatch):
     s = MID
     w = synth.gen_weights(s, seed=8)
     prompts = synth.gen_prompts(3, 121, s.V, seed=2).numpy()  # 61 pairs: chunks of 42 rows (14 positions)
+    monkeypatch.setenv("PIPO_PREFILL_ATTN", "rows")
     a = _prefill_state(s, w, prompts, 42)
     monkeypatch.setenv("PIPO_PREFILL_ATTN", "tile")
     b = _prefill_state(s, w, prompts, 42)
@@ -107,7 +127,6 @@ def test_chunked_equals_position_by_position(regular):
     assert list(a[4][0]) == list(b[4][0])  # cache lengths
 
 
-ONE = "prefill=one position at a time"
 TILES, ROWS = "prefill=chunks of %d rows (attn_prefill_kernel)", "prefill=chunks of %d rows (per-row attention)"
 
 
@@ -154,11 +173,10 @@ def test_batches_above_128_keep_the_products_of_their_steps(rows):
             assert np.array_equal(Ka, Kb) and np.array_equal(Va, Vb)
 
 
-@pytest.mark.parametrize("attn", ["rows", "tile"])
-def test_chunked_regular_prefill_matches_oracle(monkeypatch, attn):
-    monkeypatch.setenv("PIPO_PREFILL_ROWS", "64")
-    if attn == "tile":
-        monkeypatch.setenv("PIPO_PREFILL_ATTN", "tile")
+@pytest.mark.parametrize("rows,attn", [(64, "rows"), (64, "tile"), (0, "rows")])
+def test_chunked_regular_prefill_matches_oracle(monkeypatch, rows, attn):
+    monkeypatch.setenv("PIPO_PREFILL_ROWS", str(rows))
+    monkeypatch.setenv("PIPO_PREFILL_ATTN", attn)
     s = MID
     w = synth.gen_weights(s, seed=6)
     B, T = 2, 90  # 89 positions in chunks of 32, 32, 25, then the last
@@ -167,6 +185,7 @@ def test_chunked_regular_prefill_matches_oracle(monkeypatch, attn):
     try:
         orc = O.State(O.Model(s, w, max_ctx=T + 6), B)
         tok, _ = g.regular_prefill(prompts)
+        assert (KERNEL[attn] if rows else ONE) in g.describe()
         o = orc.regular_prefill(prompts)
         tol = tol_for(s)
         for step in range(5):
@@ -189,12 +208,11 @@ def test_chunked_prefill_4b(monkeypatch, attn):
     """The 4B shapes of the benchmark: a 300-token prompt (150 pairs) in
     chunks of 128 rows at B = 1, then forced-replay steps, against the oracle."""
     monkeypatch.setenv("PIPO_PREFILL_ROWS", "128")
-    if attn == "tile":
-        monkeypatch.setenv("PIPO_PREFILL_ATTN", "tile")
+    monkeypatch.setenv("PIPO_PREFILL_ATTN", attn)
     s = synth.B4
     w = synth.gen_weights(s, seed=0, device="cuda")
     host = {k: v.cpu() for k, v in w.items()}
     prompts = synth.gen_prompts(1, 300, s.V, seed=3).numpy()
-    st = run_forced_replay(s, w, prompts, 3, oracle_weights=host)
+    st = run_forced_replay(s, w, prompts, 3, oracle_weights=host, expect=KERNEL[attn])
     assert st.tok_checked >= 0.8 * st.tok_total
     del w

@@ -26,9 +26,9 @@ def test_residual_compressor_tiny_fp32():
 @pytest.mark.parametrize("B", [1, 4])
 @pytest.mark.parametrize("rows", [0, 32])
 def test_residual_compressor_bf16(monkeypatch, B, rows):
-    if rows:
-        monkeypatch.setenv("PIPO_PREFILL_ROWS", str(rows))
+    monkeypatch.setenv("PIPO_PREFILL_ROWS", str(rows))
     w = synth.gen_weights(MID, seed=3)
     prompts = synth.gen_prompts(B, 61, MID.V, seed=4).numpy()
-    st = run_forced_replay(MID, w, prompts, 6)
+    st = run_forced_replay(MID, w, prompts, 6,
+                           expect=f"chunks of {rows} rows" if rows else "one position at a time")
     assert st.tok_checked >= 0.5 * st.tok_total
