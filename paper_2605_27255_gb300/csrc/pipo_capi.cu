@@ -656,6 +656,13 @@ bool tc_prep_forced() {
     return ev && ev[0] == '1';
 }
 
+// Kernel-level calls of 33 to 64 rows on CTA pairs, the form of a step
+// (PIPO_OP_PAIR64=1, for tests; alone it is slower, see launch_gemm_tc).
+bool op_pair64() {
+    const char* ev = getenv("PIPO_OP_PAIR64");
+    return ev && ev[0] == '1';
+}
+
 // Widest batch width that runs the fused form.  Measured on the 4B shapes:
 // fused ahead at BH 16 (B = 4: 3.08 -> 2.84 ms, B = 16: 3.29 -> 2.86 ms per
 // step), behind at BH 64 (5.02 -> 5.33 ms), where the fp32 activation tile
@@ -832,7 +839,7 @@ pipo_status launch_gemm_tc(pipo_ctx* ctx, const GemvParams& p, bf16* xb, int spl
     // 35.4 / 29.4, down 28.1 / 24.9; 64 rows 15.3 / 17.5, 12.7 / 14.4, 25.8 / 25.8,
     // 19.4 / 22.8; but inside a step, where the pairs' start overlaps the launch
     // before, 64 rows are ahead too (six 4B-wide layers 1.147 -> 1.121 ms)
-    if (p.epi != EPI_ARGMAX && (bn == kPairMidN || (bn == 64 && !ctx->op_call)))
+    if (p.epi != EPI_ARGMAX && (bn == kPairMidN || (bn == 64 && (!ctx->op_call || op_pair64()))))
         return launch_gemm_pair_mid(ctx, p, xb, bn, splits_req);
     void* args[] = {&tmW, &tmX, &tp};
     ctx->prof_kind = 0;

@@ -48,6 +48,23 @@ def test_gemm_tc_matches_float64(mode, N, K, B, splits):
     assert err <= 2e-5 * scale * max(1.0, K / 1024) + 1e-6, (err, scale)
 
 
+@pytest.mark.parametrize("mode,N,K", [(0, 2560, 9728), (1, 1333, 2560), (0, 333, 4096), (1, 64, 64), (0, 128, 576),
+                                      (0, 40000, 64)])
+@pytest.mark.parametrize("B", [33, 50, 64])
+@pytest.mark.parametrize("splits", [0, 1, 2, 4])
+def test_pair_kernel_of_64_rows_matches_float64(monkeypatch, mode, N, K, B, splits):
+    """gemm_pair_mid_kernel<64>, the form that steps of 33 to 64 sequences
+    take, at the edges of its split: one K block and 152, fewer blocks than
+    splits, a ragged last row tile, more row tiles than resident pairs."""
+    a, ref = _run_tc(mode, N, K, B, splits)
+    monkeypatch.setenv("PIPO_OP_PAIR64", "1")
+    y, ref = _run_tc(mode, N, K, B, splits)
+    # more than eight K blocks to a split: sums by segments, so in other bits, so another kernel ran
+    assert K < 2560 or not torch.equal(a, y)
+    scale = ref.abs().max().item() + 1e-6
+    assert (y - ref).abs().max().item() <= 2e-5 * scale * max(1.0, K / 1024) + 1e-6
+
+
 def test_gemm_tc_split_orders_agree():
     """Different K splits change only the fp32 summation order."""
     a, ref = _run_tc(0, 2560, 9728, 16, 1)
