@@ -1,22 +1,26 @@
-"""CPU checks of the index and fragment arithmetic of two kernels, restated in
+"""CPU checks of the index and fragment arithmetic of three kernels, restated in
 numpy (no GPU):
 
-* the causal tile attention (attn_prefill_kernel): the 128-byte-swizzled K/V
-  tile layout, the ldmatrix addressing, the m16n8k16 fragment layouts of the
+* the causal tile attention (attn_prefill_kernel): the swizzled images of
+  queries, keys and values in shared memory, the operands that its
+  shared-memory descriptors (K-major for Q and K, MN-major for V) and its TMEM
+  columns (probabilities) name, the bf16 part and remainder of queries and
+  probabilities, the causal mask, the copied groups of the last tile and the
+  order in which the output is rescaled, against direct attention;
+* the sampler's selection (sample_kernel): packed keys, a warp's k best by
+  repeated maxima, the merge of the warps' lists, the slices of 4096 logits and
+  the rounds of the last CTA, against a sorted reference, with ties and small
+  vocabularies;
+* the decode attention (attn_mma_kernel): the m16n8k16 fragment layouts of the
   PTX ISA (A row g / g+8 in registers a0..a3, B column g, accumulator rows g
-  and g+8), the bf16 hi / lo split of the queries in rows 0-7 / 8-15 and of
-  the probabilities, the causal mask and the output recombination, against
-  direct attention on one 16-entry group;
-* the sampler's selection (sample_kernel): per-thread sorted top lists,
-  k warp-merge rounds with owner hand-off, the warp-0 merge of the warp
-  lists, against a sorted reference, with ties and small vocabularies;
-* the decode attention's stage rings (attn_mma_kernel, 10 and 20 stages):
-  per-warp stage ownership and the mbarrier phase parities.
+  and g+8) and ldmatrix addressing, of scores and of the value product (on
+  eight queries), and its stage rings (10 and 20 stages): per-warp stage
+  ownership and the mbarrier phase parities.
 """
 import numpy as np
 
 
-# ---- tile attention ------------------------------------------------------
+# ---- bf16 parts and the decode attention's tiles -----------------------------
 
 def _bf16(x):
     x = np.asarray(x, np.float32)
@@ -131,70 +135,159 @@ def test_tile_attention_fragment_arithmetic():
         assert np.abs(out[i] - ref).max() < 1e-4, i
 
 
+# ---- tile attention ------------------------------------------------------
+
+PF_HALF = 128 * 128  # bytes of 64 dims of 128 rows
+
+
+def _swz(addr):  # the 128-byte swizzle: 16-byte chunk (bits 4-6) by row of 128 bytes (bits 7-9)
+    return addr ^ (((addr >> 7) & 7) << 4)
+
+
+def _image(M):
+    """A tile [128][128] in shared memory as TMA boxes of 16 rows x 64 dims (K,
+    V) or the kernel's own stores (Q) leave it; a list of 2-byte slots."""
+    buf = np.full(PF_HALF, np.nan, np.float32)
+    for r in range(128):
+        for d in range(128):
+            buf[_swz((d // 64) * PF_HALF + r * 128 + (d % 64) * 2) // 2] = M[r, d]
+    return buf
+
+
+def _k_major(buf, start):
+    """Operand [128 rows][16] that umma_desc_sw128(start) names: rows 128 bytes
+    apart, groups of eight 1024."""
+    return np.array([[buf[_swz(start + (r // 8) * 1024 + (r % 8) * 128 + 2 * k) // 2] for k in range(16)]
+                     for r in range(128)])
+
+
+def _mn_major(buf, start):
+    """Operand [16 entries][128 dims] that umma_desc_mn128(start) names: 64 dims
+    in a row of 128 bytes, the next 64 PF_HALF on, groups of eight entries 1024."""
+    return np.array([[buf[_swz(start + (n // 64) * PF_HALF + (k // 8) * 1024 + (k % 8) * 128 + (n % 64) * 2) // 2]
+                      for n in range(128)] for k in range(16)])
+
+
+def test_tile_attention_operands_and_order():
+    rng = np.random.default_rng(0)
+    DH, G, C, tile, n0 = 128, 4, 45, 1, 150  # the tile of chunk positions 32 .. 44 (of 64)
+    TP = 128 // G
+    jfirst, jlast = tile * TP, min(C, (tile + 1) * TP) - 1
+    nent = n0 + jlast + 1
+    nt = -(-nent // 128)
+    assert nt == 2
+    cap = -(-nent // 16) * 16  # whole groups of the cache
+    K = _bf16(rng.standard_normal((cap, DH)).astype(np.float32))
+    V = _bf16(rng.standard_normal((cap, DH)).astype(np.float32))
+    Q = (rng.standard_normal((128, DH)) * 0.1).astype(np.float32)  # rotated, pre-scaled; row v = (position, head)
+    Q[(jlast + 1 - jfirst) * G:] = 0.0
+    q_img = [_image(_bf16(Q)), _image(_bf16(_rest(Q)))]
+    qpos = np.array([n0 + jfirst + r // G if jfirst + r // G < C else n0 + jlast for r in range(128)])
+    glast = (nent - 1) // 16
+    o = np.zeros((128, DH))
+    m_run, l_run, t_prev = np.full(128, -np.inf), np.zeros(128), None
+    for t in range(nt):
+        rows = np.concatenate([np.arange(16) + min(t * 8 + i, glast) * 16 for i in range(8)])
+        k_img, v_img = _image(K[rows]), _image(V[rows])
+        S = np.zeros((128, 128))
+        for part in range(2):
+            for k in range(DH // 16):
+                off = (k >> 2) * PF_HALF + (k & 3) * 32
+                S += _k_major(q_img[part], off).astype(np.float64) @ _k_major(k_img, off).astype(np.float64).T
+        S = np.where(t * 128 + np.arange(128)[None, :] > qpos[:, None], -np.inf, S)
+        m_new = np.maximum(m_run, S.max(1))
+        P = np.exp(S - m_new[:, None]).astype(np.float32)
+        tm = np.zeros((128, 128, 2), np.float32)  # TMEM columns of bf16 pairs: parts at 0, remainders at 64
+        for hf in range(2):
+            for i in range(32):
+                for e in range(2):
+                    p = P[:, hf * 64 + 2 * i + e]
+                    tm[:, hf * 32 + i, e], tm[:, 64 + hf * 32 + i, e] = _bf16(p), _bf16(_rest(p))
+        T = np.zeros((128, DH))
+        for part in range(2):
+            for k in range(8):
+                A = tm[:, part * 64 + k * 8:part * 64 + k * 8 + 8].reshape(128, 16)
+                T += A.astype(np.float64) @ _mn_major(v_img, k * 2048).astype(np.float64)
+        if t_prev is not None:
+            o += t_prev  # the tile before, still relative to its maximum
+        corr = np.exp(m_run - m_new)
+        l_run = l_run * corr + P.sum(1)
+        o *= corr[:, None]
+        m_run, t_prev = m_new, T
+    o = (o + t_prev) / l_run[:, None]
+    for r in range((jlast + 1 - jfirst) * G):
+        s = K[:qpos[r] + 1].astype(np.float64) @ Q[r].astype(np.float64)
+        p = np.exp(s - s.max())
+        ref = (p / p.sum()) @ V[:qpos[r] + 1].astype(np.float64)
+        assert np.abs(o[r] - ref).max() < 1e-4, r
+
+
 # ---- sampler selection ---------------------------------------------------
 
-KMAX, THREADS, WARPS = 32, 256, 8
-SENT = (-np.inf, 0x7FFFFFFF)
+KMAX, THREADS, WARPS, PER = 32, 256, 8, 16
+SLICE = THREADS * PER
 
 
-def _before(a, b):
-    return a[0] > b[0] or (a[0] == b[0] and a[1] < b[1])
+def _key(v, i):
+    """argmax_key: the value's bits in an order of unsigned integers, then the
+    lower id first."""
+    u = int((np.float32(v) + np.float32(0.0)).view(np.uint32))
+    return (((~u & 0xFFFFFFFF) if u >> 31 else u | 0x80000000) << 32) | (~i & 0xFFFFFFFF)
+
+
+def _block_select(keys, k):
+    """keys[thread][j] (0: none) -> the block's k best in order (samp_select)."""
+    lists = []
+    for w in range(WARPS):
+        mine = [list(t) for t in keys[w * 32:(w + 1) * 32]]
+        out = []
+        for _ in range(k):
+            m = max(max(t) for t in mine)
+            out.append(m)
+            if m:
+                owners = [t for t in mine if m in t]
+                assert len(owners) == 1  # keys are unique: one lane drops it
+                owners[0][owners[0].index(m)] = 0
+        lists.append(out)
+    pos, best = [0] * WARPS, []
+    for _ in range(k):
+        heads = [lists[w][pos[w]] if pos[w] < k else 0 for w in range(WARPS)]
+        m = max(heads)
+        best.append(m)
+        if m:
+            pos[heads.index(m)] += 1
+    return best
 
 
 def _select(vals, k):
     V = len(vals)
     k = min(k, V)
-    lists = []
-    for t in range(THREADS):
-        L = [SENT] * KMAX
-        for i in range(t, V, THREADS):
-            c = (float(vals[i]), i)
-            if not _before(c, L[-1]):
-                continue
-            L[-1] = c
-            for j in range(KMAX - 1, 0, -1):
-                if _before(L[j], L[j - 1]):
-                    L[j], L[j - 1] = L[j - 1], L[j]
-        lists.append(L)
-    wl = []
-    for w in range(WARPS):
-        ls = lists[w * 32:(w + 1) * 32]
-        out = []
-        for _ in range(k):
-            best = ls[0][0]
-            for l in ls[1:]:
-                if _before(l[0], best):
-                    best = l[0]
-            for l in ls:
-                if l[0] == best:
-                    l.pop(0)
-                    l.append(SENT)
-            out.append(best)
-        wl.append(out)
-    pos = [0] * 32
-    fin = []
-    for _ in range(k):
-        offers = [wl[l][pos[l]] if (l < WARPS and pos[l] < k) else SENT for l in range(32)]
-        best = offers[0]
-        for c in offers[1:]:
-            if _before(c, best):
-                best = c
-        for l in range(32):
-            if l < WARPS and pos[l] < k and offers[l] == best:
-                pos[l] += 1
-        fin.append(best)
-    return fin
+    S = -(-V // SLICE)
+    part = []
+    for s in range(S):
+        ids = [[s * SLICE + t + j * THREADS for j in range(PER)] for t in range(THREADS)]
+        part += _block_select([[_key(vals[i], i) if i < V else 0 for i in row] for row in ids], k)
+    done, best, total = 0, [], S * k
+    while True:  # the last CTA's rounds, the best so far joining the next
+        carry = k if done else 0
+        flat = best[:carry] + part[done:done + SLICE - carry]
+        flat += [0] * (SLICE - len(flat))
+        done += SLICE - carry
+        best = _block_select([[flat[t + j * THREADS] for j in range(PER)] for t in range(THREADS)], k)
+        if done >= total:
+            break
+    return [~x & 0xFFFFFFFF for x in best]
 
 
 def test_sampler_selection_is_the_sorted_top_k():
     rng = np.random.default_rng(0)
-    for trial in range(40):
-        V = int(rng.choice([5, 31, 33, 257, 600, 3001]))
+    for trial in range(24):
+        V = int(rng.choice([5, 31, 33, 257, 600, 4096, 4097, 9000]))
         k = int(rng.integers(1, 33))
         vals = rng.standard_normal(V).astype(np.float32)
         if trial % 3 == 0:
-            vals = np.round(vals * 2) / 2  # ties: the lower id first
-        ref = sorted(((float(vals[i]), i) for i in range(V)), key=lambda x: (-x[0], x[1]))[:min(k, V)]
+            vals = np.round(vals * 2) / 2  # ties (also of -0 and +0): the lower id first
+        ref = sorted(range(V), key=lambda i: (-float(vals[i]), i))[:min(k, V)]
         assert _select(vals, k) == ref, (V, k)
 
 
