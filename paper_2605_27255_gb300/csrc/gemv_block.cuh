@@ -27,7 +27,8 @@
 // Measured on the fp32 blocks H = 1024, F = 2816, B = 6 (cold, ncu): a warp per
 // (row, K slice) with the input re-read for every row took 27-56 us per
 // projection of 4-12 MB, this kernel 10.9 (gate/up, 23 MB: 36.1 -> 14.2); the
-// whole 4-layer step 804 -> 287 us.
+// whole 4-layer step 804 -> 287 us (242 now, with the gain loads below and the
+// acceptance and host changes beside it).
 //
 // bf16 weights: products are taken two along k with the paired fp32
 // instructions (the sum of eight products joins the running sum in one add

@@ -298,13 +298,7 @@ pipo_status upload_block(pipo_ctx* ctx, BlockW& bw, int l, const void* an, const
     return PIPO_OK;
 }
 
-int next_pow2_le8(int b) {
-    int nb = 1;
-    while (nb < b && nb < 8) nb <<= 1;
-    return nb;
-}
-
-// launch handles of the GEMV kernels of weight type T (k_gemv_*.cu)
+// launch handles of the CUDA-core GEMV kernels (k_gemv_*.cu)
 void* pick_block(bool bf, int ru) { return bf ? k_pick_block_bf16(ru) : k_pick_block_f32(ru); }
 template <typename T>
 void* pick_stream(int nb, int ru, bool rows) {
@@ -907,7 +901,7 @@ pipo_status launch_gemv(pipo_ctx* ctx, GemvParams p) {
     ctx->prof_bytes = (double)p.N * (two ? 2 : 1) * p.K * ctx->esz;
     if (p.B <= 4) {
         // streaming kernel: one CTA per SM, chunk-balanced, deterministic
-        int nb = std::min(4, next_pow2_le8(std::max(1, p.B)));
+        int nb = p.B <= 1 ? 1 : p.B <= 2 ? 2 : 4;  // sequences per weight pass
         while (nb > 1 && (size_t)nb * p.K * 4 + (size_t)p.K * ctx->esz > kStreamBudget) nb >>= 1;
         if ((size_t)p.K * 4 > kStreamBudget) return fail(ctx, PIPO_EINVAL, "GEMV input length %d too large", p.K);
         const bool rows = ((size_t)p.K * ctx->esz) % 512 == 0;
@@ -1747,8 +1741,8 @@ pipo_status enqueue_prefill_chunk(pipo_ctx* ctx, bool regular, int j0, int C) {
 //
 // A batch of more than 128 has fp32 products in its steps too, and more
 // sequences than a weight pass: no chunks (0), position by position.  Chunks of
-// hi and lo products were 6 to 10 times as fast there and three times as far from 64
-// bits (two 4B-wide layers, 160 sequences of 20 tokens: 73 ms and 1.4e-4
+// hi and lo products are 2.4 to 6.4 times as fast there and three times as far
+// from 64 bits (two 4B-wide layers, 160 sequences of 20 tokens: 73 ms and 1.4e-4
 // against 11 ms and 4.3e-4).
 constexpr int kChunkK = 4300;
 int prefill_chunk_rows(const pipo_ctx* ctx, int B) {
@@ -2672,7 +2666,6 @@ pipo_status op_lm_head_impl(pipo_ctx& op, int32_t dtype, const void* d_E, int32_
     p.dbg = d_logits;
     p.ld_dbg = V;
     p.B = B;
-   
     p.nseg = 1;
     p.eps = eps;
     p.seg[0] = act_seg(d_h, H, H, d_gamma);
@@ -2697,7 +2690,6 @@ pipo_status op_gemv_impl(pipo_ctx& op, int32_t dtype, int32_t mode, const void* 
     p.y = d_y;
     p.ldy = N;
     p.B = B;
-   
     p.nseg = 1;
     p.seg[0] = act_seg(d_x, K, K);
     return launch_gemv(ctx, p);

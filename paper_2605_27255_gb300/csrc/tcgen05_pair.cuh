@@ -26,7 +26,7 @@
 // give up the same way).
 //
 // Measured at R = 2048 and the 4B shapes (TFLOP/s of hi and lo products, of a
-// dense bf16 fallback peak of 1900): QKV 1422, gate/up 1583, down 992 (80 tiles
+// measured dense bf16 peak of 1883): QKV 1422, gate/up 1583, down 992 (80 tiles
 // on 76 pairs: the chunk planner avoids such heights).  Without the epilogue
 // the loop runs at 2100: the rest is TMEM reads and the output phase, during
 // which the MMAs are at most two segments ahead.  A position tile narrower
@@ -450,8 +450,8 @@ __device__ __forceinline__ void pair_mid_store(const PairMidParams& p, int row, 
     }
 }
 
-// clusters of 2 * splits CTAs; tmW boxes 64 x 128 rows, tmX boxes 64 x 128 rows
-// of the [2 * kPairMidN][K] operand
+// clusters of 2 * splits CTAs; tmW boxes 64 x 128 rows, tmX boxes 64 x NT rows
+// of the [2 NT][K] operand
 template <int NT>
 __global__ void __launch_bounds__(kPairThreads, 1)
     gemm_pair_mid_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
         __syncwarp();
     } else if (warp >= 4) {
-        // ---- epilogue: warp = (lane quadrant, 64 positions); hi and lo columns are added here
+        // ---- epilogue: warp = (lane quadrant, NT / 2 positions); hi and lo columns are added here
         const int quad = warp & 3, ph = (warp - 4) >> 2;
         const uint32_t acce_lead = map_rank(smem_u32(acce), lead);
         const uint32_t src = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ph * PW);
