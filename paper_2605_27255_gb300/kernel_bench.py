@@ -72,7 +72,7 @@ def run(name: str, batch: int, iters: int, min_bytes: float = 300e6, tc: bool = 
         gamma = torch.ones(K, dtype=torch.bfloat16, device="cuda")
 
         def launch(i):
-            if fused:  # normalised input: the converter warps inside the GEMM (batch 16 or 32)
+            if fused:  # normalised input: the converter warps inside the GEMM (batch up to 32)
                 capi.pipo_op_gemm_tc_norm(mode, Ws[i % copies].data_ptr(), N, x.data_ptr(), K, gamma.data_ptr(),
                                           0, 0, 0, 0, 1e-6, batch, y.data_ptr(), splits, base, sb, st.cuda_stream)
             else:
@@ -209,7 +209,7 @@ def main() -> None:
     ap.add_argument("--splits", type=int, default=0, help="K splits of the tensor-core GEMM (0: automatic)")
     ap.add_argument("--fused", action="store_true",
                     help="the tensor-core projection with the activation split inside the GEMM (the decode step's "
-                         "form at batch widths 16 and 32; --batch 16 or 32)")
+                         "form up to 32 sequences)")
     ap.add_argument("--step", action="store_true", help="one eager decode step of a small bf16 model")
     ap.add_argument("--ctx", type=int, default=512, help="--step: cached entries per sequence")
     ap.add_argument("--prefill", type=int, default=0, help="time a pair prefill of this many tokens per sequence")
