@@ -36,7 +36,11 @@
 // chunks load without predicates: 615 -> 450 warp instructions per task.
 // 4B gate/up, 8 rows (cold): 44.9 -> 42.0 us; a 95-token join of four such
 // layers 4893 -> 4497 us.  fp32 weights keep the single instructions (in
-// pairs the fp32 step above took 258 us against 250).
+// pairs the fp32 step above took 258 us against 250).  Their chunks hold half the
+// inputs, so that a row which one warp sums alone is a chain of K / 128
+// additions per lane: relative error 1.26e-7 at K = 4096, where chains of K / 256
+// have 1.12e-7.  Rows of kBlkLong chunks and more therefore go in two slices
+// where the warps would hold whole rows (blk_slices).
 #pragma once
 
 #include <cooperative_groups.h>
@@ -52,18 +56,21 @@ constexpr int kBlkWarps = kBlkThreads / 32;
 // tasks in flight per warp (a 16-bit task takes twice its registers when it is unpacked)
 __host__ __device__ constexpr int blk_depth(int esz) { return esz == 2 ? 2 : 3; }
 constexpr int kBlkKMax = 4096;    // inputs of one K slice
+constexpr int kBlkLong = 16;      // fp32: chunks of a row that one warp does not sum alone
 constexpr int kBlkMaxSlices = 8;  // portable cluster size
 constexpr int kBlkSeg = 128;      // row blocks per pass when the slices' sums meet in shared memory
 
 // chunks (512 weight bytes of a row) of a row of K inputs, and of the longest of KS slices
 __host__ __device__ constexpr int blk_chunks(int K, int esz) { return (K * esz + 511) / 512; }
 __host__ __device__ constexpr int blk_slice_chunks(int K, int esz, int KS) { return (blk_chunks(K, esz) + KS - 1) / KS; }
-__host__ __device__ constexpr int blk_slices(int K, int esz) {
+// slices of a row of K inputs; rows: weight rows of the launch per SM
+__host__ __device__ constexpr int blk_slices(int K, int esz, int rows) {
     const int per = kBlkKMax * esz / 512;  // chunks of the largest slice
-    return (blk_chunks(K, esz) + per - 1) / per;
+    const int KS = (blk_chunks(K, esz) + per - 1) / per;
+    // from half as many row blocks as warps on, a warp holds half of a row and more
+    return KS == 1 && esz == 4 && blk_chunks(K, esz) >= kBlkLong && rows >= kBlkRows * kBlkWarps / 2 ? 2 : KS;
 }
-__host__ __device__ constexpr size_t blk_smem(int K, int esz) {
-    const int KS = blk_slices(K, esz);
+__host__ __device__ constexpr size_t blk_smem(int K, int esz, int KS) {
     return (size_t)blk_slice_chunks(K, esz, KS) * (512 / esz) * kBlkNB * 4 + (KS > 1 ? (size_t)kBlkSeg * 32 * 4 : 0);
 }
 
@@ -115,7 +122,7 @@ __device__ __forceinline__ float4 ld4_scalar(const void* base, size_t i) {
     return make_float4(ldw<T>(base, i), ldw<T>(base, i + 1), ldw<T>(base, i + 2), ldw<T>(base, i + 3));
 }
 
-// grid: clusters of KS CTAs (KS = blk_slices(K)), any number of clusters.
+// grid: clusters of KS CTAs (KS = blk_slices), any number of clusters.
 // wide: every input, table and gain address and stride allows 4-element loads.
 template <typename T, int RU>
 __global__ void __launch_bounds__(kBlkThreads, 1) gemv_kernel(GemvParams p, int wide) {
@@ -398,10 +405,14 @@ __global__ void __launch_bounds__(kBlkThreads, 1) gemv_kernel(GemvParams p, int 
                 const int blk = head_blk[warp];
                 int ws = warp - 1;
                 while (ws >= 0 && tail_blk[ws] != blk) --ws;
-                float v = ws >= 0 ? tail_val[ws][lane] : 0.f;
+                float v = ws >= 0 ? tail_val[ws][lane] : 0.f, odd = 0.f;
                 for (int w = ws + 1; w <= warp; ++w)
-                    if (head_blk[w] == blk) v += head_val[w][lane];
-                done(blk, v);
+                    if (head_blk[w] == blk) {
+                        // fp32 rows of few chunks are split over up to eight warps: two shorter chains
+                        if (EPC == 4 && (w & 1)) odd += head_val[w][lane];
+                        else v += head_val[w][lane];
+                    }
+                done(blk, EPC == 4 ? v + odd : v);
             }
             if (KS > 1) {
                 cluster.sync();  // every slice's sums are in place

@@ -914,9 +914,9 @@ pipo_status launch_gemv(pipo_ctx* ctx, GemvParams p) {
     }
     // five sequences and more: row blocks, eight sequences per weight pass
     if ((size_t)p.K * 4 > kXsBudget) return fail(ctx, PIPO_EINVAL, "GEMV input length %d too large", p.K);
-    const int KS = blk_slices(p.K, (int)ctx->esz);
+    const int KS = blk_slices(p.K, (int)ctx->esz, (int)((long long)p.N * (two ? 2 : 1) / ctx->sms));
     void* fn = pick_block(bf, two ? 2 : 1);
-    const size_t smem = blk_smem(p.K, (int)ctx->esz);
+    const size_t smem = blk_smem(p.K, (int)ctx->esz, KS);
     int clusters = 0;
     TRY(block_clusters(ctx, fn, KS, smem, &clusters));
     int wide = gemv_wide_ok(p) ? 1 : 0;
