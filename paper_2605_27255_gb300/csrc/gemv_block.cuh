@@ -40,7 +40,8 @@
 // inputs, so that a row which one warp sums alone is a chain of K / 128
 // additions per lane: relative error 1.26e-7 at K = 4096, where chains of K / 256
 // have 1.12e-7.  Rows of kBlkLong chunks and more therefore go in two slices
-// where the warps would hold whole rows (blk_slices).
+// where the warps would hold whole rows (blk_slices): 1.09e-7, at 40000 x 4096
+// 112 us against 108 (383 with the kernel before this one).
 #pragma once
 
 #include <cooperative_groups.h>
